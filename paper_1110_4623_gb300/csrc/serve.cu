@@ -8,10 +8,11 @@
 // link, or managed memory placed in device memory, which the host writes in place and the
 // admitters poll through L2.  Inside one co-resident
 // launch:
-//   * admitter blocks wait on the admission semaphore (n = number of in-flight slots), take
-//     the next request index under the ring's ticket lock, wait for that entry to appear,
-//     claim a free slot and publish the request in it (generation-tagged chunk counter,
-//     release store of the slot state);
+//   * admitter blocks admit a batch of requests at a time, one per warp: they wait on the
+//     admission semaphore (n = number of in-flight slots) for a permit each, take the batch's
+//     request indices with one acquisition of the ring's ticket lock, and each warp waits for its
+//     entry to appear, claims a free slot and publishes the request in it (generation-tagged
+//     chunk counter, release store of the slot state);
 //   * every other block claims chunks of any active slot (compare-and-swap on the slot's
 //     generation:chunk counter), sums the chunk's int32 values in int64, adds the partial to
 //     the slot's accumulator; the block that finishes a request's last chunk writes the result
@@ -28,6 +29,7 @@
 #include <string.h>
 #include <unistd.h>
 
+#include <algorithm>
 #include <atomic>
 #include <chrono>
 #include <thread>
@@ -79,10 +81,12 @@ struct Args {
   uint32_t* admit_sem;       // gsync semaphore (WINDOW), n = nslots
   Slot* slots;
   uint32_t* active_mask;     // one bit per slot (nslots <= 64)
+  unsigned long long* busy;  // one bit per slot that a lane has claimed and no worker has freed yet
   uint32_t* stats;           // [0] admitted, [32] chunks, [64] completed (own lines)
   uint32_t* status;
   unsigned long long* trace;  // optional per-request timestamps (4 per request)
   uint32_t nslots, admitters, chunk_elems;
+  uint32_t lanes;            // admission lanes per admitter block (warps 0 .. lanes - 1)
   uint64_t timeout_ns;
 };
 
@@ -182,6 +186,149 @@ __device__ bool claim_chunk(Slot* slot, uint32_t& chunk, uint32_t& gen, bool& la
   }
 }
 
+// Barrier over the admission lanes' warps of an admitter block (its other warps have left).
+__device__ __forceinline__ void lanes_sync(uint32_t lanes) {
+  __syncwarp();
+  asm volatile("barrier.sync 1, %0;" ::"r"(lanes * 32u) : "memory");
+}
+
+// Takes `n` permits of the ticket-window semaphore at once (n at most its count): n tickets in
+// a row, entered when the last of them is admitted.  Tickets are admitted in order, so at
+// most one caller holds some of its permits while it waits for the others.
+__device__ __forceinline__ int window_wait_many(const gsync::SemRef& s, uint32_t n) {
+  const uint32_t last = ptx::atom_add_relaxed(s.word(1), n) + n - 1u;
+  gsync::Waiter w;
+  uint32_t turn = ptx::ld_acquire(s.word(2));
+  while (!gsync::after(turn + s.n, last)) {
+    if (int rc = w.tick(s.timeout_ns, s.abort_word())) return rc;
+    const uint32_t ahead = last - (turn + s.n) + 1u;
+    if (s.bo.min_ns && ahead < 0x80000000u) {
+      const uint32_t ns = ahead * s.bo.min_ns;
+      __nanosleep(ns < s.bo.max_ns ? ns : s.bo.max_ns);
+    }
+    turn = ptx::ld_acquire(s.word(2));
+  }
+  return GSYNC_OK;
+}
+__device__ __forceinline__ void window_post_many(const gsync::SemRef& s, uint32_t n) {
+  ptx::red_add_release(s.word(2), n);
+}
+
+// Thread 0 of an admitter: a permit and a ring index for each lane, or false to stop.
+__device__ __forceinline__ bool take_indices(const Args& a, const gsync::SemRef& sem, const gsync::MutexRef& lock,
+                                             uint32_t& head) {
+  if (ptx::ld_relaxed(a.dev_shutdown)) return false;
+  const int rc = window_wait_many(sem, a.lanes);
+  if (rc != GSYNC_OK) {
+    record_status(a.status, rc);
+    return false;
+  }
+  if (ptx::ld_relaxed(a.dev_shutdown)) {  // pass the permits on so blocked admitters exit too
+    window_post_many(sem, a.lanes);
+    return false;
+  }
+  // The ring lock's tickets are handed out in order from 0, one per acquisition, so ticket t
+  // stands for the indices t * lanes .. + lanes - 1: the holder needs no head word and releases
+  // the lock at once.
+  const gsync::Token t = gsync::mutex_lock_thread<GSYNC_MUTEX_TICKET>(lock);
+  if (t.status != GSYNC_OK) {
+    record_status(a.status, t.status);
+    return false;
+  }
+  // The lock hands on nothing but the ticket itself, so its release needs no fence.
+  ptx::st_relaxed(lock.turn(), t.ticket + 1u);
+  head = t.ticket * a.lanes;
+  return true;
+}
+
+// Claims a slot whose bit is clear in the busy word, h mod nslots if that one is free.  The atomic
+// that sets a bit also returns the word, so a lane that loses a bit picks its next one from there
+// (a walk over the slots' own state words pays a round trip for each busy slot it meets).  The
+// permit guarantees a free slot, but not which, so this only ends without one at the deadline.
+constexpr uint32_t kNoSlot = 0xFFFFFFFFu;
+__device__ __forceinline__ uint32_t claim_slot(const Args& a, uint32_t h) {
+  const uint64_t all = a.nslots == 64u ? ~0ull : (1ull << a.nslots) - 1ull;
+  uint32_t s = h % a.nslots;
+  uint64_t deadline = 0;
+  for (;;) {
+    const uint64_t bit = 1ull << s;
+    uint64_t old;
+    asm volatile("atom.acquire.gpu.global.or.b64 %0, [%1], %2;" : "=l"(old) : "l"(a.busy), "l"(bit) : "memory");
+    if (!(old & bit)) return s;
+    uint64_t free;
+    while ((free = ~old & all) == 0) {  // the permit came before the slot's bit: it is on its way
+      const uint64_t now = ptx::globaltimer();
+      if (deadline == 0) deadline = now + a.timeout_ns;
+      if (now > deadline) return kNoSlot;
+      old = ptx::ld_relaxed_u64((const uint64_t*)a.busy);
+    }
+    // The r-th free bit, r by the request: lanes that lost the same bit part ways here (the next
+    // free bit for all of them sent a batch's lanes at one bit again and again, 7.3 us to publish
+    // a request under load against 1.9).
+    uint32_t r = h % (uint32_t)__popcll(free);
+    while (r--) free &= free - 1u;
+    s = (uint32_t)__ffsll((long long)free) - 1u;
+  }
+}
+__device__ __forceinline__ void free_slot(const Args& a, uint32_t s) {
+  asm volatile("red.release.gpu.global.and.b64 [%0], %1;" ::"l"(a.busy), "l"(~(1ull << s)) : "memory");
+}
+
+// One lane: waits for ring entry h (seq == seq_check == h + 1), claims a free slot and
+// publishes the request in it.  False to stop (shutdown, or a wait that ran out).
+__device__ __forceinline__ bool admit(const Args& a, const gsync::SemRef& sem, uint32_t h) {
+  const gsync_serve_req* e = (const gsync_serve_req*)((const char*)a.ring + (size_t)(h & a.ring_mask) * kRingStride);
+  uint4 v;
+  uint32_t polls = 0;
+  const uint64_t t0 = ptx::globaltimer();
+  for (;;) {
+    v = ld_acquire_sys_v4(e);
+    if (v.x == h + 1u && v.w == h + 1u) break;
+    if ((++polls & 15u) == 0) {
+      bool stop = false;
+      if (ld_acquire_sys(a.shutdown)) {
+        ptx::st_release(a.dev_shutdown, 1u);
+        stop = true;
+      } else if (ptx::globaltimer() - t0 > a.timeout_ns * 16 * a.lanes) {
+        // the bound of one entry's wait, for each of the batch that a lane may wait behind
+        record_status(a.status, GSYNC_ETIMEDOUT);
+        stop = true;
+      }
+      if (stop) {  // the permit goes back so that admitters blocked on it can see shutdown
+        gsync::sem_post_thread<GSYNC_SEM_WINDOW>(sem);
+        return false;
+      }
+    }
+  }
+  const uint32_t req_len = v.y, req_off = v.z, req_id = h;
+  if (a.trace) a.trace[4ull * req_id] = ptx::globaltimer();
+  const uint32_t s = claim_slot(a, h);
+  if (s == kNoSlot) {
+    record_status(a.status, GSYNC_ETIMEDOUT);
+    return false;
+  }
+  Slot* sl = &a.slots[s];
+  // gen, nchunks and the chunk counter are read (and the counter added to) by workers
+  // at any time, so they are written with strong (relaxed) stores; the rest is read
+  // only after the release of state = 2.
+  const uint32_t gen = ptx::ld_relaxed(&sl->gen) + 1u;
+  const uint32_t nch = (req_len + a.chunk_elems - 1u) / a.chunk_elems;
+  // state and gen change in one store: a worker never sees the new generation in a free slot
+  ptx::st_relaxed_u64((uint64_t*)&sl->state, 1ull | ((uint64_t)gen << 32));
+  sl->id = req_id;
+  sl->off = (int64_t)req_off;
+  sl->len = (int64_t)req_len;
+  ptx::st_relaxed(&sl->nchunks, nch == 0 ? 1u : nch);
+  sl->acc = 0ull;
+  sl->done_chunks = 0u;
+  ptx::st_relaxed(&sl->next_chunk, (gen & 0xFFFFu) << 16);
+  ptx::st_release(&sl->state, 2u);
+  for (uint32_t m = 0; m < kMaskCopies; ++m) atomicOr(&a.active_mask[32u * m + (s >> 5)], 1u << (s & 31));
+  ptx::red_add_relaxed(a.stats, 1u);
+  if (a.trace) a.trace[4ull * req_id + 1] = ptx::globaltimer();
+  return true;
+}
+
 __global__ void __launch_bounds__(kThreads) serve_kernel(Args a) {
   const uint32_t tid = threadIdx.x;
   const gsync::MutexRef lock = gsync::mutex_attach(a.ring_lock);
@@ -194,79 +341,25 @@ __global__ void __launch_bounds__(kThreads) serve_kernel(Args a) {
   uint64_t idle_since = 0;
 
   if (admitter) {
-    // Admitters: semaphore -> ring index (ticket lock) -> wait for that entry -> slot.  The
-    // permit and the index are taken before the request exists, so its arrival only waits
-    // for one read of host memory.  Thread 0 does everything; the block only idles.
-    if (tid == 0) {
-      for (;;) {
-        if (ptx::ld_relaxed(a.dev_shutdown)) break;
-        int rc = gsync::sem_wait_thread<GSYNC_SEM_WINDOW>(sem);
-        if (rc != GSYNC_OK) { record_status(a.status, rc); break; }
-        if (ptx::ld_relaxed(a.dev_shutdown)) {  // pass the permit on so blocked admitters exit too
-          gsync::sem_post_thread<GSYNC_SEM_WINDOW>(sem);
-          break;
-        }
-        // The ring's head index is the ticket of the ring lock: tickets are handed out in
-        // order from 0, one per acquisition, so the holder needs no head word and releases
-        // the lock at once.
-        const gsync::Token t = gsync::mutex_lock_thread<GSYNC_MUTEX_TICKET>(lock);
-        if (t.status != GSYNC_OK) { record_status(a.status, t.status); break; }
-        const uint32_t h = t.ticket;
-        gsync::mutex_unlock_thread<GSYNC_MUTEX_TICKET>(lock, t.ticket);
-        // wait for entry h (seq == seq_check == h + 1) or shutdown
-        const gsync_serve_req* e =
-            (const gsync_serve_req*)((const char*)a.ring + (size_t)(h & a.ring_mask) * kRingStride);
-        uint4 v;
-        uint32_t polls = 0;
-        bool stop = false;
-        const uint64_t t0 = ptx::globaltimer();
-        for (;;) {
-          v = ld_acquire_sys_v4(e);
-          if (v.x == h + 1u && v.w == h + 1u) break;
-          if ((++polls & 15u) == 0) {
-            if (ld_acquire_sys(a.shutdown)) {
-              ptx::st_release(a.dev_shutdown, 1u);
-              stop = true;
-              break;
-            }
-            if (ptx::globaltimer() - t0 > a.timeout_ns * 16) { record_status(a.status, GSYNC_ETIMEDOUT); stop = true; break; }
-          }
-        }
-        if (stop) {  // the permit goes back so that admitters blocked on it can see shutdown
-          gsync::sem_post_thread<GSYNC_SEM_WINDOW>(sem);
-          break;
-        }
-        const uint32_t req_len = v.y, req_off = v.z, req_id = h;
-        if (a.trace) a.trace[4ull * req_id] = ptx::globaltimer();
-        // claim a free slot (the permit guarantees one)
-        uint32_t s = h % a.nslots;
-        bool got = false;
-        for (uint32_t k = 0; k < 4u * a.nslots; ++k) {
-          if (ptx::atom_cas_acquire(&a.slots[s].state, 0u, 1u) == 0u) { got = true; break; }
-          if (++s == a.nslots) s = 0;
-        }
-        if (!got) { record_status(a.status, GSYNC_ETIMEDOUT); break; }
-        Slot* sl = &a.slots[s];
-        // gen, nchunks and the chunk counter are read (and the counter added to) by workers
-        // at any time, so they are written with strong (relaxed) stores; the rest is read
-        // only after the release of state = 2.
-        const uint32_t gen = ptx::ld_relaxed(&sl->gen) + 1u;
-        const uint32_t nch = (req_len + a.chunk_elems - 1u) / a.chunk_elems;
-        ptx::st_relaxed(&sl->gen, gen);
-        sl->id = req_id;
-        sl->off = (int64_t)req_off;
-        sl->len = (int64_t)req_len;
-        ptx::st_relaxed(&sl->nchunks, nch == 0 ? 1u : nch);
-        sl->acc = 0ull;
-        sl->done_chunks = 0u;
-        ptx::st_relaxed(&sl->next_chunk, (gen & 0xFFFFu) << 16);
-        ptx::st_release(&sl->state, 2u);
-        for (uint32_t m = 0; m < kMaskCopies; ++m) atomicOr(&a.active_mask[32u * m + (s >> 5)], 1u << (s & 31));
-        ptx::red_add_relaxed(a.stats, 1u);
-        if (a.trace) a.trace[4ull * req_id + 1] = ptx::globaltimer();
-      }
+    // Admitters: semaphore -> ring indices (ticket lock) -> wait for those entries -> slots.
+    // The permits and the indices are taken before the requests exist, so an arrival only
+    // waits for one read of host memory.  A block admits `lanes` requests at a time, lane w
+    // (thread 0 of warp w) the w-th of them.  What bounds a backlog is the ring lock's chain of
+    // hand-offs: with one acquisition per request it took 0.83 us a request whatever the number
+    // of admitters or the sizes; now one acquisition hands out a batch of indices.
+    __shared__ uint32_t s_head;
+    __shared__ int s_taken, s_left;  // written before one barrier each, and not again before the next
+    const uint32_t lane = tid >> 5;
+    if (lane >= a.lanes) return;
+    if (tid == 0) s_left = 0;
+    for (;;) {
+      if (tid == 0) s_taken = take_indices(a, sem, lock, s_head) ? 1 : 0;
+      lanes_sync(a.lanes);
+      if (!s_taken) return;
+      if ((tid & 31u) == 0u && !admit(a, sem, s_head + lane)) s_left = 1;
+      lanes_sync(a.lanes);
+      if (s_left) return;
     }
-    return;
   }
 
   // Workers: claim chunks of active slots until shutdown.
@@ -332,7 +425,8 @@ __global__ void __launch_bounds__(kThreads) serve_kernel(Args a) {
         if (a.trace) a.trace[4ull * id + 3] = ptx::globaltimer();
         st_relaxed_sys_s64(a.res + id, total);
         st_release_sys(a.done + id, 1u);
-        ptx::st_release(&sl->state, 0u);
+        ptx::st_relaxed(&sl->state, 0u);
+        free_slot(a, s_slot);
         gsync::sem_post_thread<GSYNC_SEM_WINDOW>(sem);
         ptx::red_add_relaxed(a.stats + 64, 1u);
       }
@@ -534,10 +628,14 @@ extern "C" int gsync_serve_run(const gsync_serve_cfg* cfg, gsync_serve_buffers* 
   a.active_mask = mask;
   a.stats = stats;
   a.status = status;
+  a.busy = (unsigned long long*)(status + 16);  // the status line's second half
   a.trace = (unsigned long long*)buf->trace;
   a.nslots = (uint32_t)cfg->nslots;
   a.admitters = (uint32_t)cfg->admitters;
   a.chunk_elems = (uint32_t)cfg->chunk_elems;
+  // As many lanes as the permits cover with every admitter waiting for a full batch, up to one
+  // per warp; one lane where there are fewer slots than admitters.
+  a.lanes = (uint32_t)std::max(1, std::min(kThreads / 32, cfg->nslots / cfg->admitters));
   a.timeout_ns = cfg->timeout_ns ? cfg->timeout_ns : 2000000000ull;
   if (int rc = launch_coresident(serve_kernel, cfg->nblocks, kThreads, 1, 0, st, a)) return rc;
 
