@@ -13,10 +13,11 @@
 //     request indices with one acquisition of the ring's ticket lock, and each warp waits for its
 //     entry to appear, claims a free slot and publishes the request in it (generation-tagged
 //     chunk counter, release store of the slot state);
-//   * every other block claims chunks of any active slot (compare-and-swap on the slot's
-//     generation:chunk counter), sums the chunk's int32 values in int64, adds the partial to
-//     the slot's accumulator; the block that finishes a request's last chunk writes the result
-//     and a completion flag into pinned host memory, frees the slot and posts the semaphore.
+//   * every other block claims chunks of any active slot (fetch-and-add on the slot's
+//     generation:chunk counter), sums the chunks' int32 values in int64 until the request has
+//     none left to hand out, and adds its partial to the slot's accumulator; the block that
+//     finishes a request writes the result and a completion flag into pinned host memory,
+//     frees the slot and posts the semaphore.
 // Requests that arrive while others run are admitted as slots free up and their chunks run
 // side by side with older requests' chunks.  Every wait is bounded (the object timeouts, or
 // the loop's own deadline) and the host's shutdown word ends the loop.
@@ -54,6 +55,9 @@ static_assert(__BYTE_ORDER__ == __ORDER_LITTLE_ENDIAN__, "the entry halves are p
 // The active mask is kept in kMaskCopies copies on separate lines (set and cleared in all,
 // read from one per worker) to spread the workers' polling.
 constexpr uint32_t kMaskCopies = 4;
+// Active slots from which a worker goes on with the chunks of the request it has: at 1e6 req/s
+// about seven requests are in flight, a drained backlog keeps most slots active.
+constexpr int kBacklog = 8;
 
 struct Slot {  // one 128-byte line; the first 16 bytes are everything a chunk claim reads
   uint32_t state;       // 0 free, 1 claimed by an admitter, 2 active
@@ -106,15 +110,18 @@ __device__ __forceinline__ uint4 ld_acquire_sys_v4(const void* p) {
 __device__ __forceinline__ void st_release_sys(uint32_t* p, uint32_t v) {
   asm volatile("st.release.sys.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
+__device__ __forceinline__ void st_relaxed_sys(uint32_t* p, uint32_t v) {
+  asm volatile("st.relaxed.sys.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
 __device__ __forceinline__ void st_relaxed_sys_s64(int64_t* p, int64_t v) {
   asm volatile("st.relaxed.sys.global.s64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-// Block-wide int64 sum of pool[a, b): 16-byte streaming loads over the aligned middle, eight
-// of them in flight per thread (issued before any is added; the last, partial pass -- every
-// request's last chunk -- too, with the loads past the end predicated off), scalars at the
-// ends.
-__device__ __forceinline__ long long block_sum(const int32_t* pool, int64_t a, int64_t b) {
+// This thread's share of the int64 sum of pool[a, b): 16-byte streaming loads over the aligned
+// middle, eight of them in flight per thread (issued before any is added; the last, partial
+// pass -- every request's last chunk -- too, with the loads past the end predicated off),
+// scalars at the ends.
+__device__ __forceinline__ long long thread_sum(const int32_t* pool, int64_t a, int64_t b) {
   constexpr int kInFlight = 8;
   long long s = 0;
   int64_t a4 = (a + 3) & ~(int64_t)3;
@@ -143,6 +150,11 @@ __device__ __forceinline__ long long block_sum(const int32_t* pool, int64_t a, i
     for (int k = 0; k < kInFlight; ++k) s += (long long)x[k].x + x[k].y + x[k].z + x[k].w;
   }
   for (int64_t i = b4 + threadIdx.x; i < b; i += blockDim.x) s += pool[i];
+  return s;
+}
+
+// Sum of the threads' shares, valid in thread 0.
+__device__ __forceinline__ long long block_reduce(long long s) {
   __shared__ long long red[kThreads / 32];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
@@ -152,30 +164,33 @@ __device__ __forceinline__ long long block_sum(const int32_t* pool, int64_t a, i
   if (threadIdx.x == 0)
     for (uint32_t w = 0; w < (blockDim.x + 31) / 32; ++w) t += red[w];
   __syncthreads();
-  return t;  // valid in thread 0
+  return t;
 }
 
 __device__ __forceinline__ bool gen_after(uint32_t a, uint32_t b) { return (int16_t)(uint16_t)(a - b) > 0; }
 
-// Thread 0: claims one chunk of slot s, or returns false.  The claim is one fetch-and-add on
-// the slot's (generation:16 | chunk:16) counter, so racing workers each get a distinct chunk
-// in one round trip.  A result past the generation's chunk count is an over-claim and is
-// dropped (a request has at most 32767 chunks, so over-claims never reach the generation
-// bits).  A claim that lands after the slot moved to a newer request is a real chunk of that
-// request: the worker waits (bounded) for the newer generation to be published and serves
-// it.  A claim of an older generation than the one now published is dropped.
-__device__ bool claim_chunk(Slot* slot, uint32_t& chunk, uint32_t& gen, bool& last, uint64_t timeout_ns) {
+// Thread 0: claims one chunk of slot s, or returns false.  A look at the slot comes first: only
+// one that is active with chunks left is worth a claim.  The claim is one fetch-and-add on the
+// slot's (generation:16 | chunk:16) counter, so racing workers each get a distinct chunk in one
+// round trip.  A claim of the generation that the look saw needs no second look: its chunk
+// count stands until the request completes, which this chunk holds up.  A result past the
+// generation's chunk count is an over-claim and is dropped (a request has at most 32767 chunks,
+// so over-claims never reach the generation bits).  A claim that lands after the slot moved to
+// a newer request is a real chunk of that request: the worker waits (bounded) for the newer
+// generation to be published and serves it.  A claim of an older generation than the one now
+// published is dropped.
+__device__ bool claim_chunk(Slot* slot, uint32_t& chunk, uint32_t& nchunks, uint64_t timeout_ns) {
+  uint4 h = gsync::ptx::ld_acquire_v4(&slot->state);
+  if (h.x != 2u || (h.z >> 16) != (h.y & 0xFFFFu) || (h.z & 0xFFFFu) >= h.w) return false;
   const uint32_t v = gsync::ptx::atom_add_relaxed(&slot->next_chunk, 1u);
   const uint32_t g = v >> 16, c = v & 0xFFFFu;
   uint64_t deadline = 0;
   for (;;) {
-    const uint4 h = gsync::ptx::ld_acquire_v4(&slot->state);
     const uint32_t hg = h.y & 0xFFFFu;
     if (h.x == 2u && hg == g) {
       if (c >= h.w) return false;
       chunk = c;
-      gen = h.y;
-      last = c + 1u == h.w;
+      nchunks = h.w;
       return true;
     }
     if (gen_after(hg, g) || (hg == g && h.x != 2u && h.x != 1u)) return false;  // stale claim
@@ -183,6 +198,7 @@ __device__ bool claim_chunk(Slot* slot, uint32_t& chunk, uint32_t& gen, bool& la
     const uint64_t now = ptx::globaltimer();
     if (deadline == 0) deadline = now + timeout_ns;
     if (now > deadline) return false;
+    h = gsync::ptx::ld_acquire_v4(&slot->state);
   }
 }
 
@@ -270,8 +286,15 @@ __device__ __forceinline__ uint32_t claim_slot(const Args& a, uint32_t h) {
     s = (uint32_t)__ffsll((long long)free) - 1u;
   }
 }
+
+// After a fence that orders the request's last use of the slot.
 __device__ __forceinline__ void free_slot(const Args& a, uint32_t s) {
-  asm volatile("red.release.gpu.global.and.b64 [%0], %1;" ::"l"(a.busy), "l"(~(1ull << s)) : "memory");
+  asm volatile("red.relaxed.gpu.global.and.b64 [%0], %1;" ::"l"(a.busy), "l"(~(1ull << s)) : "memory");
+}
+// The slot's last chunk is handed out: it has no more work to find, so it leaves the active
+// mask (it cannot be reused before that chunk completes).
+__device__ __forceinline__ void retire_slot(const Args& a, uint32_t s) {
+  for (uint32_t k = 0; k < kMaskCopies; ++k) atomicAnd(&a.active_mask[32u * k + (s >> 5)], ~(1u << (s & 31)));
 }
 
 // One lane: waits for ring entry h (seq == seq_check == h + 1), claims a free slot and
@@ -329,15 +352,15 @@ __device__ __forceinline__ bool admit(const Args& a, const gsync::SemRef& sem, u
   return true;
 }
 
-__global__ void __launch_bounds__(kThreads) serve_kernel(Args a) {
+// Three blocks per SM: the largest grid the registers have always allowed.
+__global__ void __launch_bounds__(kThreads, 3) serve_kernel(Args a) {
   const uint32_t tid = threadIdx.x;
   const gsync::MutexRef lock = gsync::mutex_attach(a.ring_lock);
   const gsync::SemRef sem = gsync::sem_attach(a.admit_sem);
-  __shared__ int s_cmd;       // 0 continue, 1 exit
-  __shared__ uint32_t s_slot;
-  __shared__ int64_t s_lo, s_hi;
+  __shared__ int s_cmd;             // 0 work, 1 exit, 2 nothing yet
+  __shared__ int64_t s_lo[2], s_hi[2];  // the chunk to sum, and the next one (lo = hi: no more)
   const bool admitter = blockIdx.x < a.admitters;
-  uint32_t idle = 0, scan = blockIdx.x % a.nslots;
+  uint32_t idle = 0;
   uint64_t idle_since = 0;
 
   if (admitter) {
@@ -362,36 +385,44 @@ __global__ void __launch_bounds__(kThreads) serve_kernel(Args a) {
     }
   }
 
-  // Workers: claim chunks of active slots until shutdown.
+  // Workers: claim chunks of active slots until shutdown.  Thread 0 keeps the request's slot,
+  // chunk count and value range.
+  uint32_t seek = blockIdx.x * 0x85EBCA6Bu, slot = 0;
+  Slot* sl = nullptr;
+  uint32_t nchunks = 0, chunk = 0;
+  bool backlog = false;
+  int64_t off = 0, end = 0;
+  auto set_chunk = [&](uint32_t c, uint32_t k) {
+    const int64_t lo = off + (int64_t)c * a.chunk_elems;
+    s_lo[k] = lo;
+    s_hi[k] = lo + a.chunk_elems < end ? lo + a.chunk_elems : end;
+  };
   for (;;) {
     if (tid == 0) {
       s_cmd = 2;  // nothing yet
       const uint32_t* my_mask = a.active_mask + 32u * (blockIdx.x % kMaskCopies);
       uint64_t mask;  // both mask words in one load (the copy starts a line)
       asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(mask) : "l"(my_mask) : "memory");
-      // Visit only the set bits, in the order scan, scan + 1, ..., nslots - 1, 0, ..., scan - 1
-      // (bits at or above `scan` first): a walk over all slots with a division per step costs a
-      // single thread ~10 us, which every idle worker would pay whenever any slot is active.
-      const uint64_t upper = mask & (~0ull << scan), lower = mask & ~(~0ull << scan);
+      // Visit only the set bits, from a place that differs from block to block and from look to
+      // look, so that the workers spread over the active slots (all of them going on from the
+      // slot they last served, they met at the next set bit and left most slots waiting).
+      seek += 0x9E3779B1u;
+      const uint32_t from = seek >> 26;
+      const uint64_t upper = mask & (~0ull << from), lower = mask & ~(~0ull << from);
       bool got = false;
       for (int pass = 0; pass < 2 && !got; ++pass) {
         for (uint64_t m = pass ? lower : upper; m && !got; m &= m - 1u) {
           const uint32_t s = (uint32_t)__ffsll((long long)m) - 1u;
-          uint32_t c, g;
-          bool last;
-          if (!claim_chunk(&a.slots[s], c, g, last, a.timeout_ns)) continue;
-          // The last chunk is handed out: the slot has no more work to find, so it leaves the
-          // active mask now (it cannot be reused before this chunk completes).
-          if (last)
-            for (uint32_t k = 0; k < kMaskCopies; ++k) atomicAnd(&a.active_mask[32u * k + (s >> 5)], ~(1u << (s & 31)));
-          Slot* sl = &a.slots[s];
-          const int64_t lo = sl->off + (int64_t)c * a.chunk_elems;
-          int64_t hi = lo + a.chunk_elems;
-          if (hi > sl->off + sl->len) hi = sl->off + sl->len;
-          s_slot = s; s_lo = lo; s_hi = hi;
-          if (a.trace && c == 0) a.trace[4ull * sl->id + 2] = ptx::globaltimer();
+          if (!claim_chunk(&a.slots[s], chunk, nchunks, a.timeout_ns)) continue;
+          if (chunk + 1u == nchunks) retire_slot(a, s);
+          sl = &a.slots[s];
+          off = sl->off;
+          end = off + sl->len;
+          set_chunk(chunk, 0);
+          if (a.trace && chunk == 0) a.trace[4ull * sl->id + 2] = ptx::globaltimer();
           s_cmd = 0;
-          scan = s;
+          slot = s;
+          backlog = __popcll((long long)mask) >= kBacklog;
           got = true;
         }
       }
@@ -413,21 +444,50 @@ __global__ void __launch_bounds__(kThreads) serve_kernel(Args a) {
     const int cmd = s_cmd;
     if (cmd == 1) break;
     if (cmd == 2) { __syncthreads(); continue; }
-    const long long part = block_sum(a.pool, s_lo, s_hi);
+    // With a backlog, chunks of this request until they are all handed out, added up in registers:
+    // one reduction and one count of done chunks per block and request (with few requests in
+    // flight other blocks are free, and a chunk taken early would only wait here).  Thread 0 asks
+    // for the next one
+    // before it sums its share of this one, so the claim's round trip passes under the loads.
+    // No other request can take the slot meanwhile (this block's chunks are not counted done),
+    // so the claim needs no look at the slot's state, and a claim past the last chunk ends it.
+    long long sum = 0;
+    uint32_t taken = 0;
+    for (uint32_t k = 0;; k ^= 1u) {
+      uint32_t v = 0xFFFFu;
+      if (tid == 0 && backlog && chunk + 1u < nchunks) v = ptx::atom_add_relaxed(&sl->next_chunk, 1u);
+      sum += thread_sum(a.pool, s_lo[k], s_hi[k]);
+      ++taken;
+      if (tid == 0) {
+        chunk = v & 0xFFFFu;
+        if (chunk + 1u == nchunks) retire_slot(a, slot);
+        if (chunk < nchunks) set_chunk(chunk, k ^ 1u);
+        else s_lo[k ^ 1u] = s_hi[k ^ 1u] = 0;
+      }
+      __syncthreads();
+      if (s_lo[k ^ 1u] == s_hi[k ^ 1u]) break;
+    }
+    const long long part = block_reduce(sum);
     if (tid == 0) {
-      Slot* sl = &a.slots[s_slot];
-      atomicAdd(&sl->acc, (unsigned long long)part);
-      ptx::red_add_relaxed(a.stats + 32, 1u);
-      const uint32_t d = ptx::atom_add_acq_rel(&sl->done_chunks, 1u) + 1u;
-      if (d == sl->nchunks) {
-        const long long total = (long long)atomicAdd(&sl->acc, 0ull);
+      ptx::red_add_relaxed(a.stats + 32, taken);
+      long long total = part;
+      bool finished = taken == nchunks;  // the whole request: nothing to add up with other blocks
+      if (!finished) {
+        atomicAdd(&sl->acc, (unsigned long long)part);
+        finished = ptx::atom_add_acq_rel(&sl->done_chunks, taken) + taken == nchunks;
+        if (finished) total = (long long)ptx::ld_relaxed_u64((const uint64_t*)&sl->acc);
+      }
+      if (finished) {
         const uint32_t id = sl->id;
         if (a.trace) a.trace[4ull * id + 3] = ptx::globaltimer();
         st_relaxed_sys_s64(a.res + id, total);
-        st_release_sys(a.done + id, 1u);
+        // One fence for everything this block hands on: the result and its flag to the host, the
+        // slot to the next request, the permit to an admitter.
+        asm volatile("fence.acq_rel.sys;" ::: "memory");
+        st_relaxed_sys(a.done + id, 1u);
         ptx::st_relaxed(&sl->state, 0u);
-        free_slot(a, s_slot);
-        gsync::sem_post_thread<GSYNC_SEM_WINDOW>(sem);
+        free_slot(a, slot);
+        ptx::red_add_relaxed(sem.word(2), 1u);  // the ticket window's post
         ptx::red_add_relaxed(a.stats + 64, 1u);
       }
     }
@@ -443,7 +503,7 @@ __global__ void __launch_bounds__(kThreads) segsum_kernel(const int32_t* pool, i
   const int64_t lo = off + (int64_t)blockIdx.x * chunk_elems;
   int64_t hi = lo + chunk_elems;
   if (hi > off + len) hi = off + len;
-  const long long part = block_sum(pool, lo, hi);
+  const long long part = block_reduce(thread_sum(pool, lo, hi));
   if (threadIdx.x == 0) {
     atomicAdd(acc, (unsigned long long)part);
     const uint32_t d = ptx::atom_add_acq_rel(counter, 1u) + 1u;
