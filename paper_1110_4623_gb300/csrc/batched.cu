@@ -481,6 +481,32 @@ __global__ void batched_collect_kernel(Args a) {
   rec[1] = 0;
 }
 
+// An acquisition as its block's thread 0 needs it: what it adds, its key and the key's policy.
+struct __align__(16) Staged {
+  uint4 pol;
+  int64_t add;
+  uint32_t key;
+  uint32_t bad;  // 1: the key is out of range
+};
+constexpr uint32_t kStage = 32;  // acquisitions staged at a time, one per lane
+
+// Lane `lane` of a warp stages acquisition number base + lane of block b (of its nmine).
+__device__ __forceinline__ void stage(const Args& a, Staged* to, uint32_t b, uint32_t G, uint32_t base, uint32_t nmine,
+                                      uint32_t lane) {
+  const uint32_t j = base + lane;
+  if (j >= nmine) return;
+  const uint32_t i = b + j * G;
+  const uint32_t key = (uint32_t)a.keys[i];
+  Staged s;
+  s.add = a.adds[i];
+  s.key = key;
+  s.bad = key >= (uint32_t)a.nkeys;
+  const uint32_t cls = s.bad ? 0u : a.key_class[key];
+  const uint32_t* pol = a.policy + 4u * (cls < (uint32_t)a.nclasses ? cls : 0u);
+  s.pol = make_uint4(pol[0], pol[1], pol[2], pol[3]);
+  to[lane] = s;
+}
+
 // One crossing of the group barrier with the sampled slot check.
 template <int BKIND>
 __device__ __forceinline__ int group_cross(gsync::BarrierRef& bar, uint32_t* gslots, uint32_t gsize, uint32_t grank,
@@ -498,12 +524,13 @@ __device__ __forceinline__ int group_cross(gsync::BarrierRef& bar, uint32_t* gsl
 }
 
 // MAXT: the largest block the instantiation runs.  Eight blocks per SM leave 32 registers a
-// thread at 256 threads and 64 at 128; the 128-thread instantiation keeps thread 0's lock
-// paths out of local memory (no spills).
+// thread at 256 threads and 64 at 128; the 128-thread instantiation keeps thread 0's lock paths
+// out of local memory (no spills; every acquire empties L1, so a spill is an L2 round trip).
 template <int BKIND, int MAXT>
 __global__ void __launch_bounds__(MAXT, 8) batched_kernel(Args a) {
   const uint32_t G = gridDim.x, b = blockIdx.x, tid = threadIdx.x;
   __shared__ int s_fail;
+  __shared__ Staged staged[2][kStage];
   if (tid == 0) s_fail = 0;
   // The cluster cohort lock's local locks (one per key below kLocalKeys; block 0 of each
   // cluster holds the ones in use).  Initialised before any block of the cluster can use them,
@@ -560,22 +587,33 @@ __global__ void __launch_bounds__(MAXT, 8) batched_kernel(Args a) {
   const uint32_t nacq = (uint32_t)a.nacq;
   const uint32_t nmine = b < nacq ? (nacq - 1u - b) / G + 1u : 0u;
   const uint32_t rounds = g >= 0 ? (uint32_t)a.rounds : 0u;
-  uint32_t crossed = 0, mix = 0, bad = 0;
+  uint32_t crossed = 0, due = 0, mix = 0, bad = 0;
   int bar_rc = GSYNC_OK;
   __syncthreads();
+  // Acquisitions are staged kStage at a time into shared memory, by the block's last warp while
+  // thread 0 works through the batch before (by its only warp in between where there is one).
+  // Key, class and policy are three loads that depend on one another, and every lock's acquire
+  // empties L1: one after another on thread 0 they took longer than an uncontended lock.  With
+  // no key much hotter than the rest a launch is that much shorter (36 K acquisitions of 2713
+  // keys, Zipf 0.42, 152 blocks: 507 -> 374 us); a launch bound by its hottest key's chain of
+  // hand-offs is not (1e6 of 4096, Zipf 1.1, 1184 blocks: 39.1 ms before and after).
+  const uint32_t stager = (blockDim.x >> 5) - 1u;
+  if ((tid >> 5) == stager) stage(a, staged[0], b, G, 0u, nmine, tid & 31u);
   for (uint32_t j = 0; j < nmine; ++j) {
+    if ((j & (kStage - 1u)) == 0u) {
+      __syncthreads();  // batch j / kStage is there, and the one before it is used up
+      if ((tid >> 5) == stager)
+        stage(a, staged[(j / kStage + 1u) & 1u], b, G, j + kStage, nmine, tid & 31u);
+    }
     if (tid == 0 && !s_fail) {
-      const uint32_t i = b + j * G;
-      const uint32_t key = (uint32_t)a.keys[i];
-      // The addend is this block's own input: read it before the lock, so that its load (from
-      // DRAM on a launch's first touch) overlaps the wait instead of lengthening the section.
-      const int64_t add = a.adds[i];
-      if (key >= (uint32_t)a.nkeys) {
+      const Staged& it = staged[(j / kStage) & 1u][j & (kStage - 1u)];
+      const uint32_t key = it.key;
+      const int64_t add = it.add;
+      if (it.bad) {
         ptx::atom_or_relaxed(a.status, GSYNC_STATUS_VIOLATION);
         s_fail = 1;
       } else {
-        const uint32_t cls = a.key_class[key];
-        const uint32_t* pol = a.policy + 4u * (cls < (uint32_t)a.nclasses ? cls : 0u);
+        const uint32_t* pol = &it.pol.x;
         if (pol[0] == GSYNC_BATCHED_TICKET_CARRY || pol[0] == GSYNC_BATCHED_COHORT_CARRY ||
             pol[0] == GSYNC_BATCHED_CLUSTER_CARRY || pol[0] == GSYNC_BATCHED_CLUSTER_DIE_CARRY) {
           int rc;
@@ -614,16 +652,24 @@ __global__ void __launch_bounds__(MAXT, 8) batched_kernel(Args a) {
           record_status(a.status, t.status);
           s_fail = 1;
         } else {
-          a.sum[key] += add;
-          a.count[key] += 1u;
+          // both loads before either store: one round trip (a ticket lock's launch of 2e5, Zipf 0.6,
+          // 592 blocks: 3.88 -> 3.46 ms)
+          const int64_t sum0 = a.sum[key];
+          const uint32_t count0 = a.count[key];
+          a.sum[key] = sum0 + add;
+          a.count[key] = count0 + 1u;
           unlock_by_policy(m, t);
         }
         }
       }
     }
+    // The crossings are spread evenly: after acquisition j, (j + 1) * rounds / nmine of them are
+    // made, counted by carrying the remainder (a 64-bit division here, on thread 0 between two
+    // acquisitions, took as long as an L2 round trip).
     if (rounds) {
-      const uint32_t target = (uint32_t)(((uint64_t)(j + 1u) * rounds) / nmine);
-      while (crossed < target) {
+      due += rounds;
+      while (due >= nmine) {
+        due -= nmine;
         const int rc = group_cross<BKIND>(bar, gslots, gsize, grank, crossed++, mix, bad);
         if (bar_rc == GSYNC_OK) bar_rc = rc;
       }
