@@ -1,4 +1,5 @@
-"""The spin semaphores, whose posts fence before they swap: exact final state at the edges."""
+"""The CAS spin lock on both sides of the grid from which its attempts are paced, and the spin
+semaphores whose posts fence before they swap: exact final state at the edges."""
 import numpy as np
 import pytest
 
@@ -7,6 +8,20 @@ from oracle import calc
 from paper_1110_4623_gb300 import inputs
 
 pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("nblocks,threads", [(1, 256), (660, 256), (679, 256), (680, 256), (699, 128), (1216, 256),
+                                             (2400, 64)])
+@pytest.mark.parametrize("cs_words", [0, 300])
+def test_cas_spin_exact(nblocks, threads, cs_words):
+    from paper_1110_4623_gb300 import runner
+    require_gpu()
+    delay, add = inputs.mutex_inputs(nblocks, 4, nblocks)
+    got = runner.MutexRun("cas_spin", nblocks, threads, 4, cs_words, delay, add).run()
+    want = calc.mutex_final(nblocks, 4, cs_words, add)
+    assert got["rc"] == 0 and got["status"] == 0, got["status"]
+    assert got["total"] == want["total"] and np.array_equal(got["data"], want["data"])
+    assert calc.check_grant_log(got["log"], None, nblocks, 4, fifo=False) == []
 
 
 @pytest.mark.parametrize("kind", ["spin", "spin_backoff"])
