@@ -15,7 +15,7 @@ constexpr int kMaxThreads = 256;
 // The queue's bookkeeping, guarded by the mutex (plain accesses by the holder's thread 0, the
 // whole struct in one 16-byte load and one 16-byte store: one L2 round trip per look).
 struct __align__(16) Queue {
-  uint32_t count, head, tail, capacity;
+  uint32_t count, head, tail, capacity;  // init_queue_objects writes them by this order
 };
 
 template <int MKIND>
@@ -200,14 +200,8 @@ extern "C" int gsync_bench_condvar(const gsync_condvar_work* w, const gsync_back
   Queue* q = (Queue*)p;             p += round_up(sizeof(Queue));
   uint32_t* buf = (uint32_t*)p;
   const uint64_t timeout_ns = 10000000000ull;
-  if (int rc = gsync_mutex_init(mstate, gsync_mutex_bytes(w->mutex_kind, 1), w->mutex_kind, 1, backoff, timeout_ns,
-                                stream))
+  if (int rc = init_queue_objects(w->mutex_kind, mstate, nf, ne, q, (uint32_t)w->capacity, backoff, timeout_ns, st))
     return rc;
-  if (int rc = gsync_cond_init(nf, gsync_cond_bytes(), backoff, timeout_ns, stream)) return rc;
-  if (int rc = gsync_cond_init(ne, gsync_cond_bytes(), backoff, timeout_ns, stream)) return rc;
-  const Queue q0 = {0u, 0u, 0u, (uint32_t)w->capacity};
-  GSYNC_CUDA(cudaMemcpyAsync(q, &q0, sizeof q0, cudaMemcpyHostToDevice, st));
-  GSYNC_CUDA(cudaStreamSynchronize(st));  // q0 lives on this stack frame
   const int items_per_consumer = (int)(items / w->consumers);
   auto kernel = w->mutex_kind == GSYNC_MUTEX_COHORT        ? condvar_workload_kernel<GSYNC_MUTEX_COHORT>
                 : w->mutex_kind == GSYNC_MUTEX_CLUSTER     ? condvar_workload_kernel<GSYNC_MUTEX_CLUSTER>

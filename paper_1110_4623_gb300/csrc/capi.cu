@@ -91,8 +91,9 @@ struct InitSpec {
   uint32_t die[gsync::kMaxSmIds / 4];  // packed bytes
 };
 
-__global__ void init_state_kernel(uint32_t* s, InitSpec spec) {
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < spec.nwords; i += gridDim.x * blockDim.x) {
+// Writes words first, first + step, ... of an object.
+__device__ __forceinline__ void init_words(uint32_t* s, const InitSpec& spec, uint32_t first, uint32_t step) {
+  for (uint32_t i = first; i < spec.nwords; i += step) {
     uint32_t v = 0;
     if (i < 16) v = spec.header[i];
     if (spec.die_table && i >= gsync::kDieTableWord && i < gsync::kDieTableWord + gsync::kMaxSmIds / 4)
@@ -108,6 +109,20 @@ __global__ void init_state_kernel(uint32_t* s, InitSpec spec) {
     if (spec.spin_sem_s && line == 1 && word == 0) v = spec.spin_sem_s;
     s[i] = v;
   }
+}
+
+__global__ void init_state_kernel(uint32_t* s, InitSpec spec) {
+  init_words(s, spec, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+}
+
+// Several objects in one launch, one block row each.
+constexpr int kMaxInit = 4;
+struct InitBatch {
+  uint32_t* s[kMaxInit];
+  InitSpec spec[kMaxInit];
+};
+__global__ void init_batch_kernel(InitBatch b) {
+  init_words(b.s[blockIdx.y], b.spec[blockIdx.y], blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
 int launch_init(void* state, size_t bytes, const InitSpec& spec, cudaStream_t st) {
@@ -249,6 +264,36 @@ int init_cluster_kind(uint32_t kind, void* state, size_t bytes, int budget, cons
 }
 
 }  // namespace
+
+namespace gsync_impl {
+
+int init_queue_objects(int mutex_kind, void* mutex, void* not_full, void* not_empty, void* queue, uint32_t capacity,
+                       const gsync_backoff* backoff, uint64_t timeout_ns, cudaStream_t st) {
+  if (backoff && backoff->policy > GSYNC_BACKOFF_SPIN_THEN_SLEEP) return GSYNC_EINVAL;
+  InitBatch b;
+  const bool ticket = mutex_kind == GSYNC_MUTEX_TICKET;
+  b.s[0] = (uint32_t*)mutex;
+  fill_header(b.spec[0], kPrimMutex, (uint32_t)mutex_kind, ticket ? 1u : 0u,
+              ticket ? 0u : (uint32_t)GSYNC_COHORT_DEFAULT_BUDGET, backoff, timeout_ns, 0);
+  b.spec[0].nwords = 3 * kLine / 4;
+  if (mutex_kind == GSYNC_MUTEX_COHORT)
+    if (int rc = place_on_dies(mutex, b.spec[0], st)) return rc;
+  b.s[1] = (uint32_t*)not_full;
+  fill_header(b.spec[1], kPrimCond, 0, 0, 0, backoff, timeout_ns, 0);
+  b.spec[1].nwords = (uint32_t)(gsync_cond_bytes() / 4);
+  b.s[2] = (uint32_t*)not_empty;
+  b.spec[2] = b.spec[1];
+  b.s[3] = (uint32_t*)queue;
+  memset(&b.spec[3], 0, sizeof b.spec[3]);
+  b.spec[3].header[3] = capacity;
+  b.spec[3].nwords = 4;
+  const uint32_t threads = 256;
+  init_batch_kernel<<<dim3((b.spec[0].nwords + threads - 1) / threads, kMaxInit), threads, 0, st>>>(b);
+  GSYNC_CUDA(cudaGetLastError());
+  return GSYNC_OK;
+}
+
+}  // namespace gsync_impl
 
 extern "C" {
 

@@ -99,6 +99,13 @@ int device_topology(cudaStream_t st, uint8_t* die_of_sm, int* ndies, int* sms);
 int line_homes(const void* base, int nlines, size_t stride, const uint8_t* die_of_sm, int sms, cudaStream_t st,
                uint8_t* die_out);
 
+// The condition-variable queue's objects, written by one launch: the mutex (TICKET, COHORT,
+// CLUSTER or CLUSTER_MCS, its default budget), the two condition variables and the queue's four
+// words {0, 0, 0, capacity}.  Asynchronous but for COHORT, which measures where its lines live.
+// (Three launches, a copy and a wait for it took 20 of the 26 us of a call with no items.)
+int init_queue_objects(int mutex_kind, void* mutex, void* not_full, void* not_empty, void* queue, uint32_t capacity,
+                       const gsync_backoff* backoff, uint64_t timeout_ns, cudaStream_t st);
+
 // Maps a device-side wait result onto the caller's status bits.
 __device__ __forceinline__ void record_status(uint32_t* status, int rc) {
   if (rc == GSYNC_OK || status == nullptr) return;
