@@ -58,7 +58,63 @@ __device__ __forceinline__ void cs_store(uint32_t* data, uint32_t cs_words, uint
   }
 }
 
-template <int KIND, bool WIDE>
+// A section of many words a thread takes a pass of kCsInFlight of them, a round trip under the lock,
+// after another.  Where its data starts on a 16-byte boundary it goes through shared memory
+// instead: kStageVecs 16-byte vectors a thread at a time, asked for by cp.async (which needs no
+// registers to hold what is in flight, so that eight blocks of 256 threads still fit an SM),
+// vector j on thread j mod blockDim, each thread working on what it asked for itself; the last
+// one to three words go as in the narrow section.
+constexpr uint32_t kStageVecs = 4;
+struct StagedSection {
+  uint32_t slot;  // this thread's first vector in shared memory (shared-window address)
+  __device__ __forceinline__ void ask(const uint32_t* data, uint32_t nvec, uint32_t base) {
+#pragma unroll
+    for (uint32_t k = 0; k < kStageVecs; ++k) {
+      const uint32_t j = base + k * blockDim.x;
+      if (j < nvec)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(slot + 16u * k * blockDim.x), "l"(data + 4u * j)
+                     : "memory");
+    }
+  }
+  __device__ __forceinline__ void load(const uint32_t* data, uint32_t n) {
+    extern __shared__ uint4 stage[];
+    slot = (uint32_t)__cvta_generic_to_shared(stage + threadIdx.x);
+    ask(data, n / 4u, threadIdx.x);
+  }
+  __device__ __forceinline__ void store(uint32_t* data, uint32_t n, uint32_t v) {
+    const uint32_t tail = (n & ~3u) + threadIdx.x;
+    uint32_t last = 0;
+    if (tail < n) last = data[tail];
+    for (uint32_t base = threadIdx.x;;) {
+      asm volatile("cp.async.wait_all;" ::: "memory");
+#pragma unroll 2
+      for (uint32_t k = 0; k < kStageVecs; ++k) {
+        const uint32_t j = base + k * blockDim.x, w = 4u * j * kGolden;
+        if (j >= n / 4u) break;
+        uint4 y;
+        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(y.x), "=r"(y.y), "=r"(y.z), "=r"(y.w)
+                     : "r"(slot + 16u * k * blockDim.x)
+                     : "memory");
+        y.x += v ^ w;
+        y.y += v ^ (w + kGolden);
+        y.z += v ^ (w + 2u * kGolden);
+        y.w += v ^ (w + 3u * kGolden);
+        reinterpret_cast<uint4*>(data)[j] = y;
+      }
+      base += blockDim.x * kStageVecs;
+      if (base >= n / 4u) break;
+      ask(data, n / 4u, base);
+    }
+    if (tail < n) data[tail] = last + (v ^ (tail * kGolden));
+  }
+};
+
+// The widths of a section: no wider than the block, up to kCsInFlight words a thread at a time,
+// or staged.
+enum Width : int { kNarrow = 0, kWide = 1, kStaged = 2 };
+
+template <int KIND, int WIDTH>
 __global__ void __launch_bounds__(kMaxThreads, 8)
     mutex_workload_kernel(uint32_t* state, int acq, int cs_words, const uint32_t* __restrict__ delay,
                           const uint32_t* __restrict__ addend, uint32_t* data, uint32_t* total, uint32_t* grant_log,
@@ -102,13 +158,24 @@ __global__ void __launch_bounds__(kMaxThreads, 8)
     }
     // ---- critical section ----
     uint32_t x[kCsInFlight];
-    if (KIND != kFrameOnly) cs_load<WIDE>(data, (uint32_t)cs_words, x);  // data and total never overlap
+    StagedSection staged;
+    if (KIND != kFrameOnly) {  // data and total never overlap
+      if (WIDTH == kStaged)
+        staged.load(data, (uint32_t)cs_words);
+      else
+        cs_load<WIDTH == kWide>(data, (uint32_t)cs_words, x);
+    }
     uint32_t seq = 0;
     if (KIND != kFrameOnly && tid == 0) {
       seq = *total;
       *total = seq + 1u;
     }
-    if (KIND != kFrameOnly) cs_store<WIDE>(data, (uint32_t)cs_words, v, x);
+    if (KIND != kFrameOnly) {
+      if (WIDTH == kStaged)
+        staged.store(data, (uint32_t)cs_words, v);
+      else
+        cs_store<WIDTH == kWide>(data, (uint32_t)cs_words, v, x);
+    }
     // ---- end of critical section ----
     if (KIND >= 0) {
       gsync::mutex_unlock<KIND>(m, t);
@@ -143,23 +210,37 @@ __global__ void __launch_bounds__(kMaxThreads, 8)
 using KernelFn = void (*)(uint32_t*, int, int, const uint32_t*, const uint32_t*, uint32_t*, uint32_t*, uint32_t*,
                           uint32_t*, uint32_t*, uint32_t*);
 
-template <bool WIDE>
+template <int WIDTH>
 KernelFn pick_width(int kind) {
   switch (kind) {
-    case GSYNC_MUTEX_CAS_SPIN: return mutex_workload_kernel<GSYNC_MUTEX_CAS_SPIN, WIDE>;
-    case GSYNC_MUTEX_CAS_BACKOFF: return mutex_workload_kernel<GSYNC_MUTEX_CAS_BACKOFF, WIDE>;
-    case GSYNC_MUTEX_TICKET: return mutex_workload_kernel<GSYNC_MUTEX_TICKET, WIDE>;
-    case GSYNC_MUTEX_SLEEP_QUEUE: return mutex_workload_kernel<GSYNC_MUTEX_SLEEP_QUEUE, WIDE>;
-    case GSYNC_MUTEX_COHORT: return mutex_workload_kernel<GSYNC_MUTEX_COHORT, WIDE>;
-    case GSYNC_MUTEX_RING: return mutex_workload_kernel<GSYNC_MUTEX_RING, WIDE>;
-    case GSYNC_MUTEX_CLUSTER: return mutex_workload_kernel<GSYNC_MUTEX_CLUSTER, WIDE>;
-    case GSYNC_MUTEX_CLUSTER_MCS: return mutex_workload_kernel<GSYNC_MUTEX_CLUSTER_MCS, WIDE>;
+    case GSYNC_MUTEX_CAS_SPIN: return mutex_workload_kernel<GSYNC_MUTEX_CAS_SPIN, WIDTH>;
+    case GSYNC_MUTEX_CAS_BACKOFF: return mutex_workload_kernel<GSYNC_MUTEX_CAS_BACKOFF, WIDTH>;
+    case GSYNC_MUTEX_TICKET: return mutex_workload_kernel<GSYNC_MUTEX_TICKET, WIDTH>;
+    case GSYNC_MUTEX_SLEEP_QUEUE: return mutex_workload_kernel<GSYNC_MUTEX_SLEEP_QUEUE, WIDTH>;
+    case GSYNC_MUTEX_COHORT: return mutex_workload_kernel<GSYNC_MUTEX_COHORT, WIDTH>;
+    case GSYNC_MUTEX_RING: return mutex_workload_kernel<GSYNC_MUTEX_RING, WIDTH>;
+    case GSYNC_MUTEX_CLUSTER: return mutex_workload_kernel<GSYNC_MUTEX_CLUSTER, WIDTH>;
+    case GSYNC_MUTEX_CLUSTER_MCS: return mutex_workload_kernel<GSYNC_MUTEX_CLUSTER_MCS, WIDTH>;
   }
   return nullptr;
 }
 
-// A critical section wider than the block runs in the kernel that batches its loads.
-KernelFn pick(int kind, bool wide) { return wide ? pick_width<true>(kind) : pick_width<false>(kind); }
+KernelFn pick(int kind, Width w) {
+  return w == kStaged ? pick_width<kStaged>(kind) : w == kWide ? pick_width<kWide>(kind) : pick_width<kNarrow>(kind);
+}
+
+// Staging a pass costs more than a wide pass, so the line between them lies where the wide section
+// would start its third: 64 threads x 2000 words run 1.75x (cohort, 148 blocks: 5.12 -> 2.93 ms)
+// and 1.28x (ticket, 592: 16.9 -> 13.2 ms), 128 x 1500 1.25x and 1.08x; with two wide passes, 128 x
+// 600, 1.00x and 0.93x.
+Width width_of(int cs_words, int block_threads, const void* data) {
+  if (cs_words <= block_threads) return kNarrow;
+  return cs_words > 2 * kCsInFlight * block_threads && aligned(data, 16) ? kStaged : kWide;
+}
+
+size_t width_smem(Width w, int block_threads) {
+  return w == kStaged ? (size_t)block_threads * kStageVecs * sizeof(uint4) : 0;
+}
 
 int check_work(const gsync_mutex_work* w) {
   if (!w || w->nblocks < 1 || w->acq < 0 || w->cs_words < 0 || w->block_threads < 32 ||
@@ -187,13 +268,16 @@ size_t round_up(size_t x) { return (x + 255) & ~(size_t)255; }
 
 namespace gsync_impl {
 int max_blocks_mutex(int kind, int block_threads, int* out) {
-  // both widths must fit: the grid limit is the smaller of the two
-  KernelFn kn = pick(kind, false), kw = pick(kind, true);
-  if (!kn || !kw) return GSYNC_EINVAL;
-  int n_narrow = 0, n_wide = 0;
-  if (int rc = max_coresident(kn, block_threads, 1, 0, &n_narrow)) return rc;
-  if (int rc = max_coresident(kw, block_threads, 1, 0, &n_wide)) return rc;
-  *out = n_narrow < n_wide ? n_narrow : n_wide;
+  // every width must fit: the grid limit is the smallest of theirs
+  int least = 1 << 30;
+  for (Width w : {kNarrow, kWide, kStaged}) {
+    KernelFn k = pick(kind, w);
+    if (!k) return GSYNC_EINVAL;
+    int n = 0;
+    if (int rc = max_coresident(k, block_threads, 1, width_smem(w, block_threads), &n)) return rc;
+    least = n < least ? n : least;
+  }
+  *out = least;
   return GSYNC_OK;
 }
 }  // namespace gsync_impl
@@ -204,9 +288,11 @@ extern "C" int gsync_bench_mutex(void* state, const gsync_mutex_work* w, void* s
   if (!w->addend || !w->total || !w->grant_log || !w->ticket || !w->count || !w->status ||
       (w->cs_words > 0 && !w->data))
     return GSYNC_EINVAL;
-  KernelFn k = pick(w->kind, w->cs_words > w->block_threads);
+  const Width width = width_of(w->cs_words, w->block_threads, w->data);
+  KernelFn k = pick(w->kind, width);
   if (!k) return GSYNC_EINVAL;
-  return launch_coresident(k, w->nblocks, w->block_threads, launch_cluster(w), 0, (cudaStream_t)stream,
+  return launch_coresident(k, w->nblocks, w->block_threads, launch_cluster(w), width_smem(width, w->block_threads),
+                           (cudaStream_t)stream,
                            (uint32_t*)state, w->acq,
                            w->cs_words, w->delay, w->addend, w->data, w->total, w->grant_log, w->ticket, w->count,
                            w->status);
@@ -292,16 +378,13 @@ extern "C" int gsync_probe_cs(int cs_words, int block_threads, int iters, void* 
   GSYNC_CUDA(cudaEventCreate(&e0));
   GSYNC_CUDA(cudaEventCreate(&e1));
   GSYNC_CUDA(cudaEventRecord(e0, st));
-  if (cs_words < 0) {  // frame only: the acquire load, barriers and release store, no body
-    mutex_workload_kernel<kFrameOnly, false><<<1, block_threads, 0, st>>>(nullptr, iters, 0, nullptr, add, data, total, log,
-                                                                  tick, count, status);
-  } else if (cs_words > block_threads) {  // the same body, and the same width, as the workload's
-    mutex_workload_kernel<kNoLock, true><<<1, block_threads, 0, st>>>(nullptr, iters, cs_words, nullptr, add, data,
-                                                                     total, log, tick, count, status);
-  } else {
-    mutex_workload_kernel<kNoLock, false><<<1, block_threads, 0, st>>>(nullptr, iters, cs_words, nullptr, add, data,
-                                                                      total, log, tick, count, status);
-  }
+  const Width width = width_of(cs_words, block_threads, data);
+  KernelFn k = cs_words < 0         ? mutex_workload_kernel<kFrameOnly, kNarrow>  // the frame, no body
+               : width == kStaged   ? mutex_workload_kernel<kNoLock, kStaged>  // the workload's body at its width
+               : width == kWide     ? mutex_workload_kernel<kNoLock, kWide>
+                                    : mutex_workload_kernel<kNoLock, kNarrow>;
+  k<<<1, block_threads, width_smem(width, block_threads), st>>>(nullptr, iters, cs_words < 0 ? 0 : cs_words, nullptr, add,
+                                                               data, total, log, tick, count, status);
   GSYNC_CUDA(cudaGetLastError());
   GSYNC_CUDA(cudaEventRecord(e1, st));
   GSYNC_CUDA(cudaEventSynchronize(e1));
