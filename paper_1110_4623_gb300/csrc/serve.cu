@@ -60,7 +60,7 @@ constexpr uint32_t kMaskCopies = 4;
 constexpr int kBacklog = 8;
 
 struct Slot {  // one 128-byte line; the first 16 bytes are everything a chunk claim reads
-  uint32_t state;       // 0 free, 1 claimed by an admitter, 2 active
+  uint32_t state;       // 0 never used, 1 claimed by an admitter, 2 published (until the next claim)
   uint32_t gen;         // bumped every time the slot takes a request
   uint32_t next_chunk;  // (gen & 0xFFFF) << 16 | next chunk to hand out
   uint32_t nchunks;
@@ -331,20 +331,20 @@ __device__ __forceinline__ bool admit(const Args& a, const gsync::SemRef& sem, u
     return false;
   }
   Slot* sl = &a.slots[s];
-  // gen, nchunks and the chunk counter are read (and the counter added to) by workers
-  // at any time, so they are written with strong (relaxed) stores; the rest is read
-  // only after the release of state = 2.
+  // The slot's first 16 bytes are read (and the chunk counter added to) by workers at any time:
+  // they change in one 16-byte store, as a worker reads them in one load, so that it never sees
+  // the new request's chunk count beside the old one's generation.  Until state = 2 a claim of
+  // the new generation waits; the rest is read only after the release of that.
   const uint32_t gen = ptx::ld_relaxed(&sl->gen) + 1u;
   const uint32_t nch = (req_len + a.chunk_elems - 1u) / a.chunk_elems;
-  // state and gen change in one store: a worker never sees the new generation in a free slot
-  ptx::st_relaxed_u64((uint64_t*)&sl->state, 1ull | ((uint64_t)gen << 32));
   sl->id = req_id;
   sl->off = (int64_t)req_off;
   sl->len = (int64_t)req_len;
-  ptx::st_relaxed(&sl->nchunks, nch == 0 ? 1u : nch);
   sl->acc = 0ull;
   sl->done_chunks = 0u;
-  ptx::st_relaxed(&sl->next_chunk, (gen & 0xFFFFu) << 16);
+  asm volatile("st.relaxed.gpu.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(&sl->state), "r"(1u), "r"(gen),
+               "r"((gen & 0xFFFFu) << 16), "r"(nch == 0 ? 1u : nch)
+               : "memory");
   ptx::st_release(&sl->state, 2u);
   for (uint32_t m = 0; m < kMaskCopies; ++m) atomicOr(&a.active_mask[32u * m + (s >> 5)], 1u << (s & 31));
   ptx::red_add_relaxed(a.stats, 1u);
@@ -482,10 +482,11 @@ __global__ void __launch_bounds__(kThreads, 3) serve_kernel(Args a) {
         if (a.trace) a.trace[4ull * id + 3] = ptx::globaltimer();
         st_relaxed_sys_s64(a.res + id, total);
         // One fence for everything this block hands on: the result and its flag to the host, the
-        // slot to the next request, the permit to an admitter.
+        // slot to the next request, the permit to an admitter.  The stores after it have no order
+        // among themselves, so none of them may touch the slot: it keeps its state, and its chunk
+        // counter, past the last chunk, tells a worker that there is nothing left.
         asm volatile("fence.acq_rel.sys;" ::: "memory");
         st_relaxed_sys(a.done + id, 1u);
-        ptx::st_relaxed(&sl->state, 0u);
         free_slot(a, slot);
         ptx::red_add_relaxed(sem.word(2), 1u);  // the ticket window's post
         ptx::red_add_relaxed(a.stats + 64, 1u);
