@@ -220,7 +220,7 @@ __device__ __forceinline__ int window_wait_many(const gsync::SemRef& s, uint32_t
     const uint32_t ahead = last - (turn + s.n) + 1u;
     if (s.bo.min_ns && ahead < 0x80000000u) {
       const uint32_t ns = ahead * s.bo.min_ns;
-      __nanosleep(ns < s.bo.max_ns ? ns : s.bo.max_ns);
+      gsync::sleep_to_poll(ns < s.bo.max_ns ? ns : s.bo.max_ns);
     }
     turn = ptx::ld_acquire(s.word(2));
   }
