@@ -21,11 +21,11 @@ namespace {
 
 constexpr int kMaxThreads = 256;
 
-// Register budget: the full-fold variant reduces three values per round (64 registers); the
-// sampled variant's flag gather keeps two 16-byte vectors in flight (42 registers).  Both
-// still fit 8 blocks of 128 threads per SM, the shape of the 1184-block workloads.
+// Register budget: the full-fold variant reduces three values per round (64 registers; 48 for the
+// exchange barrier); the sampled variant's flag gather keeps two 16-byte vectors in flight (42
+// registers).  All still fit 8 blocks of 128 threads per SM, the shape of the 1184-block workloads.
 template <int KIND, bool FULL, bool TRACE = false>
-__global__ void __launch_bounds__(kMaxThreads, FULL ? 4 : 6)
+__global__ void __launch_bounds__(kMaxThreads, !FULL ? 6 : KIND == GSYNC_BAR_EXCHANGE ? 5 : 4)
     barrier_workload_kernel(uint32_t* state, int rounds, uint32_t* slots, uint32_t* chk, uint32_t* mix_out,
                             uint32_t* bad_out, uint32_t* status, uint64_t* trace = nullptr) {
   gsync::BarrierRef bar = gsync::barrier_attach(state);
@@ -35,7 +35,8 @@ __global__ void __launch_bounds__(kMaxThreads, FULL ? 4 : 6)
     if (tid == 0) gsync::ptx::atom_or_relaxed(status, GSYNC_STATUS_CONFIG);
     return;  // uniform: every block sees the same header
   }
-  __shared__ uint32_t red_x[kMaxThreads / 32], red_s[kMaxThreads / 32], red_b[kMaxThreads / 32];
+  // FULL: each warp's share of a round's fold {xor, hash sum, mismatches, -}, by round parity.
+  __shared__ uint4 red[2][kMaxThreads / 32];
   uint32_t mix = 0, bad = 0;
   constexpr bool kExchange = KIND == GSYNC_BAR_EXCHANGE;
   // The value of slot j this round: the slot buffer, or block j's exchange record.
@@ -59,6 +60,28 @@ __global__ void __launch_bounds__(kMaxThreads, FULL ? 4 : 6)
   constexpr bool kDeferFold = !FULL && !kExchange;
   uint32_t pend_v = 0, pend_want = 0;
   bool pend = false;
+  // Full fold: a warp's share takes three reduction instructions, and thread 0 puts the warps'
+  // shares of round q together one round later, in the shadow of that round's reads, so that
+  // neither this nor the store to chk (which the next arrival's release would wait for) lies
+  // between a crossing and the next arrival.  The shares alternate by round parity; the next
+  // crossing's own block barrier comes between their writes and this.  Counting barrier, 16 blocks
+  // x 128: 1.71 -> 1.56 us a round, 150 x 256: 1.81 -> 1.58; atomic, 64 x 256: 2.22 -> 2.00.  (The
+  // next round's slot store does not go out early, beside the reads: it lands in the lines that
+  // the others are reading, 1.79 us at 16 blocks.)
+  const uint32_t fold_warps = (min(blockDim.x, B) + 31u) / 32u;  // the warps that read any slot
+  auto fold_round = [&](uint32_t q) {
+    uint32_t X = 0, S = 0, NB = 0;
+    for (uint32_t w = 0; w < fold_warps; ++w) {
+      const uint4 v = red[q & 1u][w];
+      X ^= v.x;
+      S += v.y;
+      NB += v.z;
+    }
+    chk[q * B + b] = X;
+    mix = rotl32(mix, 5) ^ S;
+    bad += NB;
+  };
+  uint32_t pend_round = 0;
   for (int r = 0; r < rounds; ++r) {
     uint32_t* buf = slots + (uint32_t)(r & 1) * B;
     const uint32_t rb = (uint32_t)r * B;
@@ -86,36 +109,49 @@ __global__ void __launch_bounds__(kMaxThreads, FULL ? 4 : 6)
     }
     if (FULL) {
       uint32_t x = 0, s = 0, nb = 0;
-      for (uint32_t j = tid; j < B; j += blockDim.x) {
-        const uint32_t v = slot(buf, j, nb);
+      auto take = [&](uint32_t j, uint32_t v) {
         x ^= v;
         s += lowbias32(v);
         nb += v != rb + j;
-      }
+      };
+      // Every value is used (so its read is done) before the block's next arrival, which lets the
+      // others write the slots again.
+      if constexpr (kExchange) {
+        if (tid == 0 && pend) fold_round(pend_round);
+        if (B <= blockDim.x) {
+          if (tid < B) take(tid, slot(buf, tid, nb));
+        } else {
+          // Several records a thread: three in flight (48 registers), and a poll only for one that does not show
+          // this crossing yet (296 blocks of 32 threads: 4.74 -> 3.97 us a round).
+          const uint64_t ge = bar.epoch_base + bar.epoch;
+          for (uint32_t j0 = tid; j0 < B; j0 += 3u * blockDim.x) {
+            uint64_t lo[3], hi[3];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        x ^= __shfl_xor_sync(0xFFFFFFFFu, x, o);
-        s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-        nb += __shfl_xor_sync(0xFFFFFFFFu, nb, o);
-      }
-      if ((tid & 31) == 0) {
-        red_x[tid >> 5] = x;
-        red_s[tid >> 5] = s;
-        red_b[tid >> 5] = nb;
-      }
-      __syncthreads();
-      if (tid == 0) {
-        const uint32_t nw = (blockDim.x + 31) / 32;
-        uint32_t X = 0, S = 0, NB = 0;
-        for (uint32_t w = 0; w < nw; ++w) {
-          X ^= red_x[w];
-          S += red_s[w];
-          NB += red_b[w];
+            for (uint32_t k = 0; k < 3u; ++k) {
+              const uint32_t j = j0 + k * blockDim.x;
+              if (j < B) gsync::ptx::ld_relaxed_b128(gsync::exchange_record(bar, ge, j), lo[k], hi[k]);
+            }
+#pragma unroll
+            for (uint32_t k = 0; k < 3u; ++k) {
+              const uint32_t j = j0 + k * blockDim.x;
+              if (j < B) take(j, lo[k] == ge ? (uint32_t)hi[k] : slot(buf, j, nb));
+            }
+          }
         }
-        chk[rb + b] = X;
-        mix = rotl32(mix, 5) ^ S;
-        bad += NB;
+      } else if (B <= blockDim.x) {
+        const uint32_t v = tid < B ? buf[tid] : 0u;
+        if (tid == 0 && pend) fold_round(pend_round);
+        if (tid < B) take(tid, v);
+      } else {
+        if (tid == 0 && pend) fold_round(pend_round);
+        for (uint32_t j = tid; j < B; j += blockDim.x) take(j, buf[j]);
       }
+      x = __reduce_xor_sync(0xFFFFFFFFu, x);
+      s = __reduce_add_sync(0xFFFFFFFFu, s);
+      nb = __reduce_add_sync(0xFFFFFFFFu, nb);
+      if ((tid & 31) == 0) red[r & 1][tid >> 5] = make_uint4(x, s, nb, 0u);
+      pend = true;
+      pend_round = (uint32_t)r;
     } else if (tid == 0) {
       const uint32_t p = (b + (uint32_t)r + 1u) % B;
       const uint32_t v = slot(buf, p, bad);
@@ -129,7 +165,10 @@ __global__ void __launch_bounds__(kMaxThreads, FULL ? 4 : 6)
       }
     }
   }
-  if (kDeferFold && tid == 0 && pend) {
+  if (FULL) {
+    __syncthreads();
+    if (tid == 0 && pend) fold_round(pend_round);
+  } else if (kDeferFold && tid == 0 && pend) {
     mix = rotl32(mix, 5) ^ lowbias32(pend_v);
     bad += pend_v != pend_want;
   }
