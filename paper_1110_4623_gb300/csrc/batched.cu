@@ -22,9 +22,15 @@ namespace {
 
 constexpr int kMaxThreads = 256;
 // Per-object memory: a mutex is a header line and two lines (lock word, turn); a group
-// barrier a header line, two arrival counters (by epoch parity) and the release epoch.
+// barrier a header line, then, without clusters, the counting barrier's counter, and in a cluster
+// launch the leaders' two arrival counters (by epoch parity) and the release epoch.
 constexpr uint32_t kMutexObjWords = 3 * gsync::kLineWords;
 constexpr uint32_t kBarObjWords = 4 * gsync::kLineWords;
+// The group barriers.  Without clusters, the counting barrier: one hand-off fewer per crossing than
+// the two-stage atomic one (296 blocks in 9 groups, 20 K acquisitions, 100 crossings: 323 -> 268 us;
+// 152 blocks, 36 K, 28: 343 -> 330).  In a cluster launch, the hardware cluster barrier and the atomic
+// one over the leaders: its counting form measured no better there (706 against 709 us).
+constexpr uint32_t kCountSleep = 8;  // ns per 16 arrivals still missing
 // Keys below this may use the cluster locks (the cluster cohort lock and the carrying locks
 // over clusters): their local locks live in a table in each block's shared memory (32 bytes a
 // key).
@@ -416,6 +422,9 @@ __device__ __forceinline__ int hier_carry_add(LocalSlot* slot, uint32_t* obj, ui
 // global record; its counters, turns and records all return to zero.
 __global__ void batched_collect_kernel(Args a) {
   const uint32_t key = blockIdx.x * blockDim.x + threadIdx.x;
+  // The groups' arrival counters return to zero, so that the next launch may have other sizes.
+  for (uint32_t g = key; !a.clustered && g < (uint32_t)a.ngroups; g += gridDim.x * blockDim.x)
+    *(uint64_t*)(a.group_state + g * kBarObjWords + 1 * gsync::kLineWords) = 0ull;
   if (key >= (uint32_t)a.nkeys) return;
   const uint32_t cls = a.key_class[key];
   const uint32_t* pol = a.policy + 4u * (cls < (uint32_t)a.nclasses ? cls : 0u);
@@ -579,10 +588,12 @@ __global__ void __launch_bounds__(MAXT, 8) batched_kernel(Args a) {
     bar.s = a.group_state + (uint32_t)g * kBarObjWords;
     bar.kind = BKIND;
     bar.n = gsize;
-    bar.param = BKIND == GSYNC_BAR_CLUSTER ? ptx::cluster_nctarank() : 0u;
+    bar.param = BKIND == GSYNC_BAR_CLUSTER ? ptx::cluster_nctarank() : kCountSleep;
     bar.mode = 0;
     bar.timeout_ns = a.timeout_ns;
-    bar.epoch = ptx::ld_relaxed(bar.line(2));
+    bar.epoch = BKIND == GSYNC_BAR_CLUSTER ? ptx::ld_relaxed(bar.line(2)) : 0u;
+    bar.base = 0;
+    bar.sub_base = 0;
   }
   const uint32_t nacq = (uint32_t)a.nacq;
   const uint32_t nmine = b < nacq ? (nacq - 1u - b) / G + 1u : 0u;
@@ -708,13 +719,13 @@ int launch_batched(const gsync_batched_work* w, int cluster, const Args& a, cuda
     // For stream capture: an ordinary launch after the same co-residency check.  All blocks
     // are resident as long as no other kernel occupies the GPU when the graph runs.
     int maxb = 0;
-    if (int rc = max_coresident(batched_kernel<GSYNC_BAR_ATOMIC, MAXT>, w->block_threads, 1, 0, &maxb)) return rc;
+    if (int rc = max_coresident(batched_kernel<GSYNC_BAR_COUNT, MAXT>, w->block_threads, 1, 0, &maxb)) return rc;
     if (w->nblocks > maxb) return GSYNC_ENOTRESIDENT;
-    batched_kernel<GSYNC_BAR_ATOMIC, MAXT><<<w->nblocks, w->block_threads, 0, st>>>(a);
+    batched_kernel<GSYNC_BAR_COUNT, MAXT><<<w->nblocks, w->block_threads, 0, st>>>(a);
     GSYNC_CUDA(cudaGetLastError());
     return GSYNC_OK;
   }
-  return launch_coresident(batched_kernel<GSYNC_BAR_ATOMIC, MAXT>, w->nblocks, w->block_threads, 1, 0, st, a);
+  return launch_coresident(batched_kernel<GSYNC_BAR_COUNT, MAXT>, w->nblocks, w->block_threads, 1, 0, st, a);
 }
 
 }  // namespace

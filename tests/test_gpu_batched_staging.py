@@ -47,3 +47,25 @@ def test_key_out_of_range_is_reported(at):
     run, _, _ = make(45 * 24, 64, 1, keys)
     got = run.run()
     assert got["rc"] == 0 and got["status"] & G.GSYNC_STATUS_VIOLATION
+
+
+def test_group_state_serves_other_groups_and_cluster_launches():
+    # One buffer of group barriers, never zeroed: launches with other group sizes and of the other
+    # kind of group barrier, one after another.
+    from paper_1110_4623_gb300 import gsync as G, runner
+    require_gpu()
+    keys, adds, _ = inputs.batched_inputs(40 * 32, NKEYS, 0.8, seed=11)
+    cls = autotune.classify_keys(keys, NKEYS, 32)
+    want = calc.batched_final(keys, adds, NKEYS)
+    state = None
+    for sizes, cluster in (([5, 9, 18], 1), ([8, 16, 8], 8), ([1, 30, 1], 1), ([16, 16], 1), ([24, 8], 8), ([7, 7, 7], 1)):
+        run = runner.BatchedRun(keys, adds, NKEYS, 32, np.array(sizes), 13, cls, 3, block_threads=64, cluster=cluster)
+        run.set_policy(POLICIES[1] if cluster == 1 else POLICIES[8])
+        if state is None:
+            state = run.group_state
+        run.work.group_state = G.ptr(state)
+        for _ in range(2):
+            got = run.run()
+            assert got["rc"] == 0 and got["status"] == 0, (sizes, got["status"])
+            assert np.array_equal(got["sum"], want["sum"]) and np.array_equal(got["count"], want["count"])
+            assert not got["bad"].any()
