@@ -1726,23 +1726,26 @@ class ServeSlot:
     """One slot of the persistent serving loop (not in the paper): an admitter publishes
     requests into the slot one after another, and workers claim the requests' chunks.
 
-    Block 0 is the admitter.  For request r it takes the free slot (compare-and-swap of the
-    state 0 -> 1), reads the generation and writes generation + 1, the chunk count NCH[r], the
-    done count 0 and the accumulator 0, resets the claim counter to (generation, chunk 0),
-    publishes the slot (state 2) and sets its bit in the active mask.  Blocks 1.. are workers.
-    A worker that finds the bit set claims with one fetch-and-add on the (generation, chunk)
-    counter, then reads (state, generation, chunk count) in one access: the claim is taken when
-    the slot is active in the claim's generation and the chunk exists, dropped when the slot
-    has moved on or the chunk is past the last, and waits while the slot is being set up.  The
-    worker that takes the last chunk clears the bit.  A taken chunk adds its value (1 << chunk)
-    to the accumulator and counts itself done; the block whose count completes the request
-    reads the accumulator, which must hold every chunk, frees the slot (state 0) and counts
-    the request completed.  Workers stop once every request is completed.  Each shared access
+    Block 0 is the admitter.  For request r it takes the free slot (sets its busy bit), writes the
+    done count 0 and the accumulator 0, then in one store state 1, generation + 1, the chunk
+    count NCH[r] and the claim counter (generation, chunk 0), publishes the slot (state 2) and
+    sets its bit in the active mask.  Blocks 1.. are workers.  A worker that finds the bit set
+    looks at (state, generation, claim counter, chunk count) in one access and leaves a slot that
+    is not published or has no chunk left; else it claims with one fetch-and-add on the
+    (generation, chunk) counter.  A claim of the generation it saw is taken when the chunk
+    exists, without a second look; one of a newer generation waits until that is published and
+    is taken or dropped by its chunk count; one of an older generation is dropped.  The worker
+    that takes the last chunk clears the bit.  A taken chunk adds its value (1 << chunk) to the
+    accumulator and counts itself done; the block whose count completes the request reads the
+    accumulator, which must hold every chunk, frees the slot (clears its busy bit; the state
+    stays) and counts the request completed.  Workers stop once every request is completed.
+    (A device worker may go on with the same request's chunks, each claimed by the same
+    fetch-and-add, and count them done together: as one chunk of their sum.)  Each shared access
     is one step (sequential consistency).  The counter's chunk field stops growing one past the
     largest chunk count (a 16-bit field on the device, which the few claims made between a
     last chunk's hand-out and the clearing of the bit cannot carry into the generation).
-    broken="no_gen_check": a worker takes any claim whose chunk exists in the active request,
-    whatever the claim's generation (a chunk is then processed twice);
+    broken="no_gen_check": a worker takes any claim whose chunk exists in the request it saw or
+    waits for, whatever the claim's generation (a chunk is then processed twice);
     broken="no_done_reset": the admitter leaves the done count of the previous request (the
     next request never completes).
     """
@@ -1755,8 +1758,8 @@ class ServeSlot:
 
     def init(self, nproc, ops):
         # shared: state, gen, nchunks, claim counter (gen, chunk), done, acc, completed, active
-        # bit, and a ghost: the (generation, chunk) pairs processed so far
-        sh = (0, 0, 0, (0, 0), 0, 0, 0, 0, frozenset())
+        # bit, a ghost: the (generation, chunk) pairs processed so far, and the busy bit
+        sh = (0, 0, 0, (0, 0), 0, 0, 0, 0, frozenset(), 0)
         return sh, tuple((0, 0, 0, 0) for _ in range(nproc))
 
     @staticmethod
@@ -1764,29 +1767,23 @@ class ServeSlot:
         return sh[:i] + (v,) + sh[i + 1:]
 
     def step(self, p, loc, sh, nproc, ops):
-        state, gen, nch, ctr, done, acc, completed, active, seen = sh
+        state, gen, nch, ctr, done, acc, completed, active, seen, busy = sh
         pc, a, b, c = loc
         put = self._put
         R = len(self.nch)
-        if p == 0:  # admitter; a = request, b = its generation
+        if p == 0:  # admitter; a = request
             if pc == 0:
-                if state != 0:
+                if busy:
                     return loc, sh, None
-                return (1, a, b, c), put(sh, 0, 1), None
+                return (1, a, 0, 0), put(sh, 9, 1), None
             if pc == 1:
-                return (2, a, gen + 1, c), sh, None
+                return (2, a, 0, 0), put(sh, 4, done if self.broken == "no_done_reset" else 0), None
             if pc == 2:
-                return (3, a, b, c), put(sh, 1, b), None
+                return (3, a, 0, 0), put(sh, 5, 0), None
             if pc == 3:
-                return (4, a, b, c), put(sh, 2, self.nch[a]), None
+                return (4, a, 0, 0), (1, gen + 1, self.nch[a], (gen + 1, 0)) + sh[4:], None
             if pc == 4:
-                return (5, a, b, c), put(sh, 4, done if self.broken == "no_done_reset" else 0), None
-            if pc == 5:
-                return (6, a, b, c), put(sh, 5, 0), None
-            if pc == 6:
-                return (7, a, b, c), put(sh, 3, (b, 0)), None
-            if pc == 7:
-                return (8, a, b, c), put(sh, 0, 2), None
+                return (5, a, 0, 0), put(sh, 0, 2), None
             a += 1
             return ((0 if a < R else DONE), a, 0, 0), put(sh, 7, 1), None
         # worker; a, b = the claim's (generation, chunk), c = the request's chunk count
@@ -1795,19 +1792,26 @@ class ServeSlot:
                 return (DONE, 0, 0, 0), sh, None
             return (10, 0, 0, 0), sh, None
         if pc == 10:
-            return ((1 if active else 0), 0, 0, 0), sh, None
+            return ((11 if active else 0), 0, 0, 0), sh, None
+        if pc == 11:  # the look: a, b = the generation and the chunk count it saw
+            if state != 2 or ctr[0] != gen or ctr[1] >= nch:
+                return (0, 0, 0, 0), sh, None
+            return (1, gen, nch, 0), sh, None
         if pc == 1:
             g, k = ctr
             # the chunk field stops at max(NCH) + 1: every claim past a request's last chunk is
             # dropped alike, and the bound keeps the state space finite
-            return (2, g, k, 0), put(sh, 3, (g, min(k + 1, max(self.nch) + 1))), None
+            sh = put(sh, 3, (g, min(k + 1, max(self.nch) + 1)))
+            if g == a or self.broken == "no_gen_check":
+                return ((3, a, k, b) if k < b else (0, 0, 0, 0)), sh, None
+            return (2, g, k, 0), sh, None
         if pc == 2:
             g, k = a, b
             if state == 2 and (gen == g or self.broken == "no_gen_check"):
                 if k >= nch:
                     return (0, 0, 0, 0), sh, None  # past the last chunk: dropped
                 return (3, gen, k, nch), sh, None
-            if gen > g or (gen == g and state == 0):
+            if gen > g:
                 return (0, 0, 0, 0), sh, None  # the slot has moved on: dropped
             return loc, sh, None  # generation g is being set up: wait
         if pc == 3:  # the last chunk handed out: the slot leaves the active mask
@@ -1825,7 +1829,7 @@ class ServeSlot:
                 return loc, sh, ("violation", f"generation {a} completed with chunks {acc:#b} of {c}")
             return (7, a, b, c), sh, None
         if pc == 7:
-            return (8, a, b, c), put(sh, 0, 0), None
+            return (8, a, b, c), put(sh, 9, 0), None
         return (0, 0, 0, 0), put(sh, 6, completed + 1), None
 
 
