@@ -18,8 +18,13 @@ struct __align__(16) Queue {
   uint32_t count, head, tail, capacity;  // init_queue_objects writes them by this order
 };
 
-template <int MKIND>
-__global__ void __launch_bounds__(kMaxThreads)
+// ROOMY: up to 48 registers a thread.  Left to itself the ticket lock's kernel takes 32, which lets
+// 2432 blocks of 128 threads be resident, and keeps some of thread 0's state in local memory: every
+// acquire empties L1, so each look at it under the lock is an L2 round trip.  The roomy form runs
+// where its smaller limit (1520) admits the grid (592 + 592 blocks 20.4 -> 19.5 ms for 5920 items,
+// 384 + 384 of 32 threads 10.45 -> 10.33, 128 + 64 6.90 -> 6.85).
+template <int MKIND, bool ROOMY = false>
+__global__ void __launch_bounds__(kMaxThreads, ROOMY ? 5 : 0)
     condvar_workload_kernel(uint32_t* mutex_state, uint32_t* nf_state, uint32_t* ne_state, Queue* q, uint32_t* buf,
                             int producers, int items_per_producer, int items_per_consumer,
                             const uint32_t* __restrict__ value, uint32_t* seen, int64_t* sum, uint32_t* count,
@@ -207,9 +212,16 @@ extern "C" int gsync_bench_condvar(const gsync_condvar_work* w, const gsync_back
                 : w->mutex_kind == GSYNC_MUTEX_CLUSTER     ? condvar_workload_kernel<GSYNC_MUTEX_CLUSTER>
                 : w->mutex_kind == GSYNC_MUTEX_CLUSTER_MCS ? condvar_workload_kernel<GSYNC_MUTEX_CLUSTER_MCS>
                                                            : condvar_workload_kernel<GSYNC_MUTEX_TICKET>;
-  return launch_coresident(kernel, w->producers + w->consumers, w->block_threads, cluster, 0, st, mstate, nf, ne, q, buf,
-                           w->producers, w->items_per_producer, items_per_consumer, w->value, w->seen, w->sum,
-                           w->count, w->status, w->acquisitions);
+  auto launch = [&](auto k) {
+    return launch_coresident(k, w->producers + w->consumers, w->block_threads, cluster, 0, st, mstate, nf, ne, q, buf,
+                             w->producers, w->items_per_producer, items_per_consumer, w->value, w->seen, w->sum,
+                             w->count, w->status, w->acquisitions);
+  };
+  if (w->mutex_kind == GSYNC_MUTEX_TICKET) {
+    const int rc = launch(condvar_workload_kernel<GSYNC_MUTEX_TICKET, true>);
+    if (rc != GSYNC_ENOTRESIDENT) return rc;
+  }
+  return launch(kernel);
 }
 
 // T_cs probe of the condition-variable queue: see condvar_cs_probe_kernel.  workspace as for
