@@ -330,9 +330,8 @@ extern "C" int gsync_bench_mutex_host(const gsync_mutex_work* w, const gsync_bac
 
   if (w->delay) GSYNC_CUDA(cudaMemcpyAsync(d_delay, w->delay, 4 * n, cudaMemcpyHostToDevice, st));
   GSYNC_CUDA(cudaMemcpyAsync(d_add, w->addend, 4 * n, cudaMemcpyHostToDevice, st));
-  if (w->cs_words) GSYNC_CUDA(cudaMemsetAsync(d_data, 0, 4 * (size_t)w->cs_words, st));
-  GSYNC_CUDA(cudaMemsetAsync(d_total, 0, 4, st));
-  GSYNC_CUDA(cudaMemsetAsync(d_status, 0, 4, st));
+  // data, total and status start at zero; they lie together (with count between them): one memset
+  GSYNC_CUDA(cudaMemsetAsync(d_data, 0, (size_t)(p - (char*)d_data), st));
   if (int rc = gsync_mutex_init(state, sb, w->kind, w->nblocks, backoff, 0, stream)) return rc;
   gsync_mutex_work dw = *w;
   dw.delay = w->delay ? d_delay : nullptr;
