@@ -464,10 +464,11 @@ constexpr uint64_t kMcsOwned = 1ull << 16;
 // takes a same-word swap each ~0.65 ns and an unloaded round trip is ~400 ns, so it is full from
 // about 620 blocks on.  A larger grid spaces each block's attempts to one per (blocks x 0.65 ns)
 // round, the unit's own pace: enough that some block tries every ns, and no queue.  1184 blocks x
-// 256 threads, 64-word section: 520 -> 890 K acquisitions/s; 900: 772 -> 938 K; 700: 895 -> 957 K.
+// 256 threads, 64-word section, 100 acquisitions each: 229 -> 145 ms (516 -> 815 K/s); 20 each: 900
+// blocks 23.3 -> 19.2 ms, 700 blocks 15.6 -> 14.6.
 // Up to 676 blocks there is no pause, and the loop is the plain one (at 592 a pause gains 1 %).
-// Spinning on a load between attempts instead lets every waiter see the lock free at once: 610 K
-// at 1184 blocks.
+// Spinning on a load between attempts instead lets every waiter see the lock free at once: 1.17x
+// at 1184 blocks where the pause gives 1.42x (30 each).
 __device__ __forceinline__ uint32_t cas_spin_pause_ns() {
   const uint32_t round_ns = gridDim.x * gridDim.y * gridDim.z / 20u * 13u;
   return round_ns > 440u ? min(round_ns - 400u, 4000u) : 0u;
