@@ -621,6 +621,12 @@ int check_requests(const gsync_serve_cfg* cfg, const gsync_serve_buffers* buf) {
   return GSYNC_OK;
 }
 
+// As many lanes as the permits cover with every admitter waiting for a full batch, up to one per
+// warp; one lane where there are fewer slots than admitters.
+uint32_t admission_lanes(const gsync_serve_cfg* cfg) {
+  return (uint32_t)std::max(1, std::min(kThreads / 32, cfg->nslots / cfg->admitters));
+}
+
 }  // namespace
 
 extern "C" size_t gsync_serve_workspace_bytes(int nslots) {
@@ -667,7 +673,11 @@ extern "C" int gsync_serve_run(const gsync_serve_cfg* cfg, gsync_serve_buffers* 
   if (int rc = ring_device_ptr(buf->ring, kRingStride * (size_t)cfg->ring_slots, st, &d_ring)) return rc;
   volatile uint32_t* ctrl = buf->ctrl;
   ctrl[32] = 0;
-  memset(buf->ring, 0, kRingStride * (size_t)cfg->ring_slots);
+  // Cleared as far as an admitter may look: the requests, and the batch that each admitter has
+  // taken past them.  (All of a 65,536-entry ring is 8 MB, 90 us of a call.)
+  const uint32_t lanes = admission_lanes(cfg);
+  const int64_t polled = (int64_t)cfg->nreq + (int64_t)cfg->admitters * lanes;
+  memset(buf->ring, 0, kRingStride * (size_t)std::min<int64_t>(cfg->ring_slots, polled));
   for (int q = 0; q < cfg->nreq; ++q) buf->done[q] = 0;
   std::atomic_thread_fence(std::memory_order_seq_cst);
 
@@ -694,9 +704,7 @@ extern "C" int gsync_serve_run(const gsync_serve_cfg* cfg, gsync_serve_buffers* 
   a.nslots = (uint32_t)cfg->nslots;
   a.admitters = (uint32_t)cfg->admitters;
   a.chunk_elems = (uint32_t)cfg->chunk_elems;
-  // As many lanes as the permits cover with every admitter waiting for a full batch, up to one
-  // per warp; one lane where there are fewer slots than admitters.
-  a.lanes = (uint32_t)std::max(1, std::min(kThreads / 32, cfg->nslots / cfg->admitters));
+  a.lanes = lanes;
   a.timeout_ns = cfg->timeout_ns ? cfg->timeout_ns : 2000000000ull;
   if (int rc = launch_coresident(serve_kernel, cfg->nblocks, kThreads, 1, 0, st, a)) return rc;
 
@@ -766,16 +774,10 @@ extern "C" int gsync_serve_run(const gsync_serve_cfg* cfg, gsync_serve_buffers* 
   collector.join();
   __atomic_store_n(&buf->ctrl[32], 1u, __ATOMIC_RELEASE);
   GSYNC_CUDA(cudaStreamSynchronize(st));
-  uint32_t hstat[4] = {0, 0, 0, 0};
-  GSYNC_CUDA(cudaMemcpy(&hstat[0], stats, 4, cudaMemcpyDeviceToHost));
-  GSYNC_CUDA(cudaMemcpy(&hstat[1], stats + 32, 4, cudaMemcpyDeviceToHost));
-  GSYNC_CUDA(cudaMemcpy(&hstat[2], stats + 64, 4, cudaMemcpyDeviceToHost));
-  GSYNC_CUDA(cudaMemcpy(&hstat[3], status, 4, cudaMemcpyDeviceToHost));
-  buf->stats[0] = hstat[0];
-  buf->stats[1] = hstat[1];
-  buf->stats[2] = hstat[2];
-  buf->stats[3] = hstat[3];
-  if (rc == GSYNC_OK && hstat[3]) rc = GSYNC_ETIMEDOUT;
+  uint32_t hstat[4 * 32];  // the three counters' lines and the status line, which follows them
+  GSYNC_CUDA(cudaMemcpy(hstat, stats, sizeof hstat, cudaMemcpyDeviceToHost));
+  for (int i = 0; i < 4; ++i) buf->stats[i] = hstat[32 * i];
+  if (rc == GSYNC_OK && hstat[3 * 32]) rc = GSYNC_ETIMEDOUT;
   return rc;
 }
 

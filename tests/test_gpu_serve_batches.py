@@ -32,3 +32,20 @@ def test_backlog_exact(pool, nslots, admitters, nreq, ring_slots):
     assert np.array_equal(r["res"], calc.serve_final(off[:nreq], ln[:nreq], p))
     chunks = int((-(-ln[:nreq] // 1024)).sum())
     assert r["stats"] == [nreq, chunks, nreq, 0]
+
+
+@pytest.mark.parametrize("first,then", [(3001, 40), (300, 299), (40, 3001)])
+def test_ring_with_an_earlier_calls_entries(pool, first, then):
+    # One ring for two calls: entries of the longer one past the shorter one's must not be taken.
+    from paper_1110_4623_gb300 import runner
+    off, ln, p, dp = pool
+    ring = None
+    for n, start in ((first, 0), (then, 5 if then < first else 0)):
+        idx = (np.arange(n) + start) % len(off)
+        r = runner.ServeRun(off[idx], ln[idx], np.zeros(n, dtype=np.int64), dp, nslots=64, nblocks=80, admitters=8,
+                            chunk_elems=1024, ring_slots=4096, drain_timeout_s=10)
+        ring = r.ring = ring if ring is not None else r.ring
+        got = r.run()
+        assert got["rc"] == 0, got["stats"]
+        assert np.array_equal(got["res"], calc.serve_final(off[idx], ln[idx], p))
+        assert got["stats"][0] == n and got["stats"][2] == n
