@@ -1727,110 +1727,125 @@ class ServeSlot:
     requests into the slot one after another, and workers claim the requests' chunks.
 
     Block 0 is the admitter.  For request r it takes the free slot (sets its busy bit), writes the
-    done count 0 and the accumulator 0, then in one store state 1, generation + 1, the chunk
-    count NCH[r] and the claim counter (generation, chunk 0), publishes the slot (state 2) and
-    sets its bit in the active mask.  Blocks 1.. are workers.  A worker that finds the bit set
-    looks at (state, generation, claim counter, chunk count) in one access and leaves a slot that
-    is not published or has no chunk left; else it claims with one fetch-and-add on the
-    (generation, chunk) counter.  A claim of the generation it saw is taken when the chunk
-    exists, without a second look; one of a newer generation waits until that is published and
-    is taken or dropped by its chunk count; one of an older generation is dropped.  The worker
+    done count 0 and the accumulator 0, publishes the claim word (chunk count NCH[r], next chunk
+    0) in one access and sets the slot's bit in the active mask.  Blocks 1.. are workers.  A
+    worker that finds the bit set looks at the claim word and leaves a slot that has no chunk
+    left; else it claims with one fetch-and-add on the word, which returns the next chunk and the
+    count of the request that it belongs to.  A claim past that count is dropped.  The worker
     that takes the last chunk clears the bit.  A taken chunk adds its value (1 << chunk) to the
-    accumulator and counts itself done; the block whose count completes the request reads the
-    accumulator, which must hold every chunk, frees the slot (clears its busy bit; the state
-    stays) and counts the request completed.  Workers stop once every request is completed.
-    (A device worker may go on with the same request's chunks, each claimed by the same
-    fetch-and-add, and count them done together: as one chunk of their sum.)  Each shared access
-    is one step (sequential consistency).  The counter's chunk field stops growing one past the
-    largest chunk count (a 16-bit field on the device, which the few claims made between a
-    last chunk's hand-out and the clearing of the bit cannot carry into the generation).
-    broken="no_gen_check": a worker takes any claim whose chunk exists in the request it saw or
-    waits for, whatever the claim's generation (a chunk is then processed twice);
+    worker's sum; with keep=True the worker goes on claiming chunks of the request, without a
+    look, until a claim is past the last.  It then adds its sum to the accumulator and counts its
+    chunks done together; the block whose count completes the request reads the accumulator,
+    which must hold every chunk, frees the slot (clears its busy bit; the claim word stays) and
+    counts the request completed.  Workers stop once every request is completed.  Each shared
+    access is one step (sequential consistency).  The next chunk stops growing one past the
+    largest chunk count, and the word also carries the request's number, which no device code has:
+    it says which request a claim was taken for.
+    broken="no_gen_check": a worker serves its claim as one of the request that its look saw
+    (a chunk is then processed twice);
     broken="no_done_reset": the admitter leaves the done count of the previous request (the
-    next request never completes).
+    next request never completes);
+    broken="torn_publish": the two halves of the claim word are published by two accesses, the
+    next chunk first (a claim between them is judged by the count of the request before);
+    broken="torn_look": a worker reads the two halves by two accesses, the count last, and takes
+    its claim's count from that look.
     """
     kind = "mutex"
     capacity = 1 << 30
     fifo = False
 
-    def __init__(self, nch=(1, 2), broken=None):
-        self.nch, self.broken = tuple(nch), broken
+    def __init__(self, nch=(1, 2), keep=False, broken=None):
+        self.nch, self.keep, self.broken = tuple(nch), keep, broken
 
     def init(self, nproc, ops):
-        # shared: state, gen, nchunks, claim counter (gen, chunk), done, acc, completed, active
-        # bit, a ghost: the (generation, chunk) pairs processed so far, and the busy bit
-        sh = (0, 0, 0, (0, 0), 0, 0, 0, 0, frozenset(), 0)
-        return sh, tuple((0, 0, 0, 0) for _ in range(nproc))
+        # shared: the claim word (request number from 1, chunk count, next chunk), done, acc,
+        # completed, active bit, a ghost: the (request, chunk) pairs processed, and the busy bit
+        sh = ((0, 0, 0), 0, 0, 0, 0, frozenset(), 0)
+        return sh, tuple((0, 0, 0, 0, 0, 0) for _ in range(nproc))
 
     @staticmethod
     def _put(sh, i, v):
         return sh[:i] + (v,) + sh[i + 1:]
 
     def step(self, p, loc, sh, nproc, ops):
-        state, gen, nch, ctr, done, acc, completed, active, seen, busy = sh
-        pc, a, b, c = loc
+        word, done, acc, completed, active, seen, busy = sh
+        pc, g, k, n, mask, lg = loc
         put = self._put
         R = len(self.nch)
-        if p == 0:  # admitter; a = request
+        idle = (0, 0, 0, 0, 0, 0)
+        if p == 0:  # admitter; g = request
+            def at(pc, g=g):
+                return (pc, g, 0, 0, 0, 0)
             if pc == 0:
                 if busy:
                     return loc, sh, None
-                return (1, a, 0, 0), put(sh, 9, 1), None
+                return at(1), put(sh, 6, 1), None
             if pc == 1:
-                return (2, a, 0, 0), put(sh, 4, done if self.broken == "no_done_reset" else 0), None
+                return at(2), put(sh, 1, done if self.broken == "no_done_reset" else 0), None
             if pc == 2:
-                return (3, a, 0, 0), put(sh, 5, 0), None
+                return at(3), put(sh, 2, 0), None
             if pc == 3:
-                return (4, a, 0, 0), (1, gen + 1, self.nch[a], (gen + 1, 0)) + sh[4:], None
+                if self.broken == "torn_publish":
+                    return at(4), put(sh, 0, (g + 1, word[1], 0)), None
+                return at(5), put(sh, 0, (g + 1, self.nch[g], 0)), None
             if pc == 4:
-                return (5, a, 0, 0), put(sh, 0, 2), None
-            a += 1
-            return ((0 if a < R else DONE), a, 0, 0), put(sh, 7, 1), None
-        # worker; a, b = the claim's (generation, chunk), c = the request's chunk count
+                return at(5), put(sh, 0, (word[0], self.nch[g], word[2])), None
+            return at(0 if g + 1 < R else DONE, g + 1), put(sh, 4, 1), None
+        # worker; g, k, n = the claim's (request, chunk, chunk count), mask = chunks in its sum,
+        # lg = the request that its look saw
         if pc == 0:
             if completed == R:
-                return (DONE, 0, 0, 0), sh, None
-            return (10, 0, 0, 0), sh, None
-        if pc == 10:
-            return ((11 if active else 0), 0, 0, 0), sh, None
-        if pc == 11:  # the look: a, b = the generation and the chunk count it saw
-            if state != 2 or ctr[0] != gen or ctr[1] >= nch:
-                return (0, 0, 0, 0), sh, None
-            return (1, gen, nch, 0), sh, None
+                return (DONE, 0, 0, 0, 0, 0), sh, None
+            return (1, 0, 0, 0, 0, 0), sh, None
         if pc == 1:
-            g, k = ctr
-            # the chunk field stops at max(NCH) + 1: every claim past a request's last chunk is
+            return ((2,) + idle[1:] if active else idle), sh, None
+        if pc == 2:  # the look
+            if self.broken == "torn_look":
+                return (9, 0, word[2], 0, 0, word[0]), sh, None
+            if word[2] >= word[1]:
+                return idle, sh, None
+            return (3, 0, 0, word[1], 0, word[0]), sh, None
+        if pc == 9:
+            return ((3, 0, 0, word[1], 0, lg) if k < word[1] else idle), sh, None
+        if pc == 3:  # the claim
+            cg, cn, ck = word
+            # the next chunk stops at max(NCH) + 1: every claim past a request's last chunk is
             # dropped alike, and the bound keeps the state space finite
-            sh = put(sh, 3, (g, min(k + 1, max(self.nch) + 1)))
-            if g == a or self.broken == "no_gen_check":
-                return ((3, a, k, b) if k < b else (0, 0, 0, 0)), sh, None
-            return (2, g, k, 0), sh, None
-        if pc == 2:
-            g, k = a, b
-            if state == 2 and (gen == g or self.broken == "no_gen_check"):
-                if k >= nch:
-                    return (0, 0, 0, 0), sh, None  # past the last chunk: dropped
-                return (3, gen, k, nch), sh, None
-            if gen > g:
-                return (0, 0, 0, 0), sh, None  # the slot has moved on: dropped
-            return loc, sh, None  # generation g is being set up: wait
-        if pc == 3:  # the last chunk handed out: the slot leaves the active mask
-            if b + 1 == c:
-                return (4, a, b, c), put(sh, 7, 0), None
-            return (4, a, b, c), sh, None
-        if pc == 4:
-            if (a, b) in seen:
-                return loc, sh, ("violation", f"chunk {b} of generation {a} processed twice")
-            return (5, a, b, c), put(put(sh, 5, acc | (1 << b)), 8, seen | {(a, b)}), None
+            sh = put(sh, 0, (cg, cn, min(ck + 1, max(self.nch) + 1)))
+            if self.broken == "no_gen_check":
+                cg, cn = lg, n
+            elif self.broken == "torn_look":
+                cn = n
+            if ck >= cn:
+                return idle, sh, None
+            return (4, cg, ck, cn, 0, 0), sh, None
+        if pc == 4:  # the last chunk handed out: the slot leaves the active mask
+            if k + 1 == n:
+                return (5, g, k, n, mask, 0), put(sh, 4, 0), None
+            return (5, g, k, n, mask, 0), sh, None
         if pc == 5:
-            return ((6 if done + 1 == c else 0), a, b, c), put(sh, 4, done + 1), None
-        if pc == 6:
-            if acc != (1 << c) - 1:
-                return loc, sh, ("violation", f"generation {a} completed with chunks {acc:#b} of {c}")
-            return (7, a, b, c), sh, None
+            if (g, k) in seen:
+                return loc, sh, ("violation", f"chunk {k} of request {g} processed twice")
+            if g > R or k >= self.nch[g - 1]:
+                return loc, sh, ("violation", f"chunk {k} of request {g}, which has no such chunk")
+            more = 6 if self.keep and k + 1 < n else 7
+            return (more, g, k, n, mask | (1 << k), 0), put(sh, 5, seen | {(g, k)}), None
+        if pc == 6:  # a further chunk of the same request, which this worker's chunks hold in place
+            cg, cn, ck = word
+            sh = put(sh, 0, (cg, cn, min(ck + 1, max(self.nch) + 1)))
+            return ((4, g, ck, n, mask, 0) if ck < n else (7, g, k, n, mask, 0)), sh, None
         if pc == 7:
-            return (8, a, b, c), put(sh, 9, 0), None
-        return (0, 0, 0, 0), put(sh, 6, completed + 1), None
+            return (8, g, k, n, mask, 0), put(sh, 2, acc | mask), None
+        if pc == 8:
+            d = done + bin(mask).count("1")
+            return ((10, g, k, n, mask, 0) if d == n else idle), put(sh, 1, d), None
+        if pc == 10:
+            if acc != (1 << n) - 1:
+                return loc, sh, ("violation", f"request {g} completed with chunks {acc:#b} of {n}")
+            return (11, g, k, n, mask, 0), sh, None
+        if pc == 11:
+            return (12, g, k, n, mask, 0), put(sh, 6, 0), None
+        return idle, put(sh, 3, completed + 1), None
 
 
 def _ghost0(model, nproc):

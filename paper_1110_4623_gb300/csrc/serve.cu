@@ -11,10 +11,10 @@
 //   * admitter blocks admit a batch of requests at a time, one per warp: they wait on the
 //     admission semaphore (n = number of in-flight slots) for a permit each, take the batch's
 //     request indices with one acquisition of the ring's ticket lock, and each warp waits for its
-//     entry to appear, claims a free slot and publishes the request in it (generation-tagged
-//     chunk counter, release store of the slot state);
-//   * every other block claims chunks of any active slot (fetch-and-add on the slot's
-//     generation:chunk counter), sums the chunks' int32 values in int64 until the request has
+//     entry to appear, claims a free slot and publishes the request in it (release store of the
+//     slot's claim word);
+//   * every other block claims chunks of any active slot (fetch-and-add on the slot's claim
+//     word), sums the chunks' int32 values in int64 until the request has
 //     none left to hand out, and adds its partial to the slot's accumulator; the block that
 //     finishes a request writes the result and a completion flag into pinned host memory,
 //     frees the slot and posts the semaphore.
@@ -59,17 +59,17 @@ constexpr uint32_t kMaskCopies = 4;
 // about seven requests are in flight, a drained backlog keeps most slots active.
 constexpr int kBacklog = 8;
 
-struct Slot {  // one 128-byte line; the first 16 bytes are everything a chunk claim reads
-  uint32_t state;       // 0 never used, 1 claimed by an admitter, 2 published (until the next claim)
-  uint32_t gen;         // bumped every time the slot takes a request
-  uint32_t next_chunk;  // (gen & 0xFFFF) << 16 | next chunk to hand out
-  uint32_t nchunks;
+struct Slot {  // one 128-byte line
+  // The claim word: chunk count << 32 | next chunk to hand out.  Only ever read, added to and
+  // published as one 64-bit word, so a claim always sees the count of the request whose chunk it
+  // took.  A slot with no request has no chunk left (never used: 0 of 0; finished: past the last).
+  uint64_t claim;
   uint32_t done_chunks;
   uint32_t id;
   int64_t off;
   int64_t len;
   unsigned long long acc;
-  uint32_t pad[20];
+  uint32_t pad[22];
 };
 static_assert(sizeof(Slot) == 128, "one line per slot");
 
@@ -167,39 +167,27 @@ __device__ __forceinline__ long long block_reduce(long long s) {
   return t;
 }
 
-__device__ __forceinline__ bool gen_after(uint32_t a, uint32_t b) { return (int16_t)(uint16_t)(a - b) > 0; }
+__device__ __forceinline__ uint64_t atom_add_acquire_u64(uint64_t* p, uint64_t v) {
+  uint64_t r;
+  asm volatile("atom.acquire.gpu.global.add.u64 %0, [%1], %2;" : "=l"(r) : "l"(p), "l"(v) : "memory");
+  return r;
+}
 
-// Thread 0: claims one chunk of slot s, or returns false.  A look at the slot comes first: only
-// one that is active with chunks left is worth a claim.  The claim is one fetch-and-add on the
-// slot's (generation:16 | chunk:16) counter, so racing workers each get a distinct chunk in one
-// round trip.  A claim of the generation that the look saw needs no second look: its chunk
-// count stands until the request completes, which this chunk holds up.  A result past the
-// generation's chunk count is an over-claim and is dropped (a request has at most 32767 chunks,
-// so over-claims never reach the generation bits).  A claim that lands after the slot moved to
-// a newer request is a real chunk of that request: the worker waits (bounded) for the newer
-// generation to be published and serves it.  A claim of an older generation than the one now
-// published is dropped.
-__device__ bool claim_chunk(Slot* slot, uint32_t& chunk, uint32_t& nchunks, uint64_t timeout_ns) {
-  uint4 h = gsync::ptx::ld_acquire_v4(&slot->state);
-  if (h.x != 2u || (h.z >> 16) != (h.y & 0xFFFFu) || (h.z & 0xFFFFu) >= h.w) return false;
-  const uint32_t v = gsync::ptx::atom_add_relaxed(&slot->next_chunk, 1u);
-  const uint32_t g = v >> 16, c = v & 0xFFFFu;
-  uint64_t deadline = 0;
-  for (;;) {
-    const uint32_t hg = h.y & 0xFFFFu;
-    if (h.x == 2u && hg == g) {
-      if (c >= h.w) return false;
-      chunk = c;
-      nchunks = h.w;
-      return true;
-    }
-    if (gen_after(hg, g) || (hg == g && h.x != 2u && h.x != 1u)) return false;  // stale claim
-    // generation g is being set up (or not yet published): wait for it, bounded
-    const uint64_t now = ptx::globaltimer();
-    if (deadline == 0) deadline = now + timeout_ns;
-    if (now > deadline) return false;
-    h = gsync::ptx::ld_acquire_v4(&slot->state);
-  }
+// Thread 0: claims one chunk of a slot, or returns false.  A look comes first: only a slot with
+// chunks left is worth a claim.  The claim is one fetch-and-add on the claim word, so racing
+// workers each get a distinct chunk in one round trip, with the chunk count of the request it
+// belongs to: of the one looked at, or of a newer one that took the slot since, and is served
+// instead.  A claim past the count is an over-claim and is dropped (the count of a later request
+// overwrites it; at most one per worker and request, far from the word's upper half).  A chunk
+// that is claimed and not yet counted done keeps the slot with its request.  The acquire belongs
+// to the claim, which reads the publication of the very request that it returns.
+__device__ __forceinline__ bool claim_chunk(Slot* slot, uint32_t& chunk, uint32_t& nchunks) {
+  const uint64_t look = ptx::ld_relaxed_u64(&slot->claim);
+  if ((uint32_t)look >= (uint32_t)(look >> 32)) return false;
+  const uint64_t v = atom_add_acquire_u64(&slot->claim, 1ull);
+  chunk = (uint32_t)v;
+  nchunks = (uint32_t)(v >> 32);
+  return chunk < nchunks;
 }
 
 // Barrier over the admission lanes' warps of an admitter block (its other warps have left).
@@ -331,21 +319,17 @@ __device__ __forceinline__ bool admit(const Args& a, const gsync::SemRef& sem, u
     return false;
   }
   Slot* sl = &a.slots[s];
-  // The slot's first 16 bytes are read (and the chunk counter added to) by workers at any time:
-  // they change in one 16-byte store, as a worker reads them in one load, so that it never sees
-  // the new request's chunk count beside the old one's generation.  Until state = 2 a claim of
-  // the new generation waits; the rest is read only after the release of that.
-  const uint32_t gen = ptx::ld_relaxed(&sl->gen) + 1u;
+  // Workers look at the claim word (and over-claims add to it) at any time, but read the rest only
+  // after a claim of this request: everything is in place before the word is published.  An
+  // over-claim of the slot's last request that lands before the publication is overwritten by it,
+  // as one after it is a chunk of this request.
   const uint32_t nch = (req_len + a.chunk_elems - 1u) / a.chunk_elems;
   sl->id = req_id;
   sl->off = (int64_t)req_off;
   sl->len = (int64_t)req_len;
   sl->acc = 0ull;
   sl->done_chunks = 0u;
-  asm volatile("st.relaxed.gpu.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(&sl->state), "r"(1u), "r"(gen),
-               "r"((gen & 0xFFFFu) << 16), "r"(nch == 0 ? 1u : nch)
-               : "memory");
-  ptx::st_release(&sl->state, 2u);
+  ptx::st_release_u64(&sl->claim, (uint64_t)(nch == 0 ? 1u : nch) << 32);
   for (uint32_t m = 0; m < kMaskCopies; ++m) atomicOr(&a.active_mask[32u * m + (s >> 5)], 1u << (s & 31));
   ptx::red_add_relaxed(a.stats, 1u);
   if (a.trace) a.trace[4ull * req_id + 1] = ptx::globaltimer();
@@ -413,7 +397,7 @@ __global__ void __launch_bounds__(kThreads, 3) serve_kernel(Args a) {
       for (int pass = 0; pass < 2 && !got; ++pass) {
         for (uint64_t m = pass ? lower : upper; m && !got; m &= m - 1u) {
           const uint32_t s = (uint32_t)__ffsll((long long)m) - 1u;
-          if (!claim_chunk(&a.slots[s], chunk, nchunks, a.timeout_ns)) continue;
+          if (!claim_chunk(&a.slots[s], chunk, nchunks)) continue;
           if (chunk + 1u == nchunks) retire_slot(a, s);
           sl = &a.slots[s];
           off = sl->off;
@@ -450,16 +434,16 @@ __global__ void __launch_bounds__(kThreads, 3) serve_kernel(Args a) {
     // for the next one
     // before it sums its share of this one, so the claim's round trip passes under the loads.
     // No other request can take the slot meanwhile (this block's chunks are not counted done),
-    // so the claim needs no look at the slot's state, and a claim past the last chunk ends it.
+    // so the claim needs no look at the slot, and a claim past the last chunk ends it.
     long long sum = 0;
     uint32_t taken = 0;
     for (uint32_t k = 0;; k ^= 1u) {
-      uint32_t v = 0xFFFFu;
-      if (tid == 0 && backlog && chunk + 1u < nchunks) v = ptx::atom_add_relaxed(&sl->next_chunk, 1u);
+      uint32_t next = nchunks;
+      if (tid == 0 && backlog && chunk + 1u < nchunks) next = (uint32_t)ptx::atom_add_relaxed_u64(&sl->claim, 1ull);
       sum += thread_sum(a.pool, s_lo[k], s_hi[k]);
       ++taken;
       if (tid == 0) {
-        chunk = v & 0xFFFFu;
+        chunk = next;
         if (chunk + 1u == nchunks) retire_slot(a, slot);
         if (chunk < nchunks) set_chunk(chunk, k ^ 1u);
         else s_lo[k ^ 1u] = s_hi[k ^ 1u] = 0;
@@ -483,8 +467,8 @@ __global__ void __launch_bounds__(kThreads, 3) serve_kernel(Args a) {
         st_relaxed_sys_s64(a.res + id, total);
         // One fence for everything this block hands on: the result and its flag to the host, the
         // slot to the next request, the permit to an admitter.  The stores after it have no order
-        // among themselves, so none of them may touch the slot: it keeps its state, and its chunk
-        // counter, past the last chunk, tells a worker that there is nothing left.
+        // among themselves, so none of them may touch the slot: its claim word, past the last
+        // chunk, tells a worker that there is nothing left.
         asm volatile("fence.acq_rel.sys;" ::: "memory");
         st_relaxed_sys(a.done + id, 1u);
         free_slot(a, slot);
