@@ -1682,7 +1682,9 @@ class RingPublish:
     (20 + i).
     broken="one_check": the admitter checks seq alone (a half of the previous lap slips in);
     broken="no_reuse_wait": the producer overwrites the slot before the admitter took the
-    previous request (that request is lost and the admitter waits forever).
+    previous request (that request is lost and the admitter waits forever);
+    broken="torn_half": the admitter reads a half by two accesses, the length before the sequence
+    number (the length of the previous lap slips in).
     """
     kind = "mutex"
     capacity = 1
@@ -1713,6 +1715,8 @@ class RingPublish:
         if pc == 0:
             return (1, i, hi if self.read_hi_first else lo), sh, None
         got_lo, got_hi = (lo, seen) if self.read_hi_first else (seen, hi)
+        if self.broken == "torn_half":
+            got_lo, got_hi = (lo[0], seen[1]), hi
         (seq, ln), (off, chk) = got_lo, got_hi
         if seq != i + 1 or (chk != i + 1 and self.broken != "one_check"):
             return (0, i, None), sh, None  # not published yet: poll again

@@ -99,13 +99,10 @@ __device__ __forceinline__ uint32_t ld_acquire_sys(const uint32_t* p) {
   asm volatile("ld.acquire.sys.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
-__device__ __forceinline__ uint4 ld_acquire_sys_v4(const void* p) {
-  uint4 v;
-  asm volatile("ld.acquire.sys.global.v4.u32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-               : "l"(p)
-               : "memory");
-  return v;
+// Two 8-byte accesses, each single-copy atomic, in no set order: the halves of a ring entry.  (A
+// vector of four words would be four accesses, and a half's number could be newer than its value.)
+__device__ __forceinline__ void ld_acquire_sys_v2(const void* p, uint64_t& lo, uint64_t& hi) {
+  asm volatile("ld.acquire.sys.global.v2.u64 {%0, %1}, [%2];" : "=l"(lo), "=l"(hi) : "l"(p) : "memory");
 }
 __device__ __forceinline__ void st_release_sys(uint32_t* p, uint32_t v) {
   asm volatile("st.release.sys.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
@@ -289,12 +286,12 @@ __device__ __forceinline__ void retire_slot(const Args& a, uint32_t s) {
 // publishes the request in it.  False to stop (shutdown, or a wait that ran out).
 __device__ __forceinline__ bool admit(const Args& a, const gsync::SemRef& sem, uint32_t h) {
   const gsync_serve_req* e = (const gsync_serve_req*)((const char*)a.ring + (size_t)(h & a.ring_mask) * kRingStride);
-  uint4 v;
+  uint64_t lo, hi;  // seq | len << 32 and off | seq_check << 32
   uint32_t polls = 0;
   const uint64_t t0 = ptx::globaltimer();
   for (;;) {
-    v = ld_acquire_sys_v4(e);
-    if (v.x == h + 1u && v.w == h + 1u) break;
+    ld_acquire_sys_v2(e, lo, hi);
+    if ((uint32_t)lo == h + 1u && (uint32_t)(hi >> 32) == h + 1u) break;
     if ((++polls & 15u) == 0) {
       bool stop = false;
       if (ld_acquire_sys(a.shutdown)) {
@@ -311,7 +308,7 @@ __device__ __forceinline__ bool admit(const Args& a, const gsync::SemRef& sem, u
       }
     }
   }
-  const uint32_t req_len = v.y, req_off = v.z, req_id = h;
+  const uint32_t req_len = (uint32_t)(lo >> 32), req_off = (uint32_t)hi, req_id = h;
   if (a.trace) a.trace[4ull * req_id] = ptx::globaltimer();
   const uint32_t s = claim_slot(a, h);
   if (s == kNoSlot) {
