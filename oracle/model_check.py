@@ -1726,6 +1726,48 @@ class RingPublish:
         return ((0 if i < ops else DONE), i, None), (lo, hi, i), None
 
 
+class RingReuse:
+    """The reuse of the serving ring's entries (the persistent serving loop; not in the paper).
+
+    Block 0 is the host's producer: it writes the `requests` requests into a ring of `entries`
+    entries, request q into entry q mod entries, once request q - entries and all before it have
+    completed.  Blocks 1.. are admission lanes: each takes the next index, waits for that index's
+    entry to appear, and completes the request, in any order among the lanes.
+    broken="completed_count": the producer goes by the number of completed requests instead, and
+    overwrites the entry of a slow lane's request when a later one completes first.
+    """
+    kind = "mutex"
+    capacity = 1
+    fifo = False
+
+    def __init__(self, entries=2, requests=4, broken=None):
+        self.entries, self.requests, self.broken = entries, requests, broken
+
+    def init(self, nproc, ops):
+        # shared: (the entries' sequence numbers, next index, requests completed)
+        return ((0,) * self.entries, 0, frozenset()), tuple((0, 0) for _ in range(nproc))
+
+    def step(self, p, loc, sh, nproc, ops):
+        pc, q = loc
+        ring, nxt, done = sh
+        if p == 0:
+            if q == self.requests:
+                return (DONE, q), sh, None
+            low = 0
+            while low in done:
+                low += 1
+            if q - (len(done) if self.broken == "completed_count" else low) >= self.entries:
+                return loc, sh, None
+            return (0, q + 1), (_set(ring, q % self.entries, q + 1), nxt, done), None
+        if pc == 0:
+            if nxt == self.requests:
+                return (DONE, q), sh, None
+            return (1, nxt), (ring, nxt + 1, done), None
+        if pc == 1:
+            return ((2 if ring[q % self.entries] == q + 1 else 1), q), sh, None
+        return (0, q), (ring, nxt, done | {q}), None
+
+
 class ServeSlot:
     """One slot of the persistent serving loop (not in the paper): an admitter publishes
     requests into the slot one after another, and workers claim the requests' chunks.

@@ -553,8 +553,9 @@ void spin_until(Clock::time_point t) {
 }
 
 // Counters shared by the host threads of a run, one per cache line: the collector updates
-// `completed` while the producer (or launcher) reads it and writes `published`, and a line
-// shared between writers on different cores would bounce on every update.
+// `completed` (how many requests) and `prefix` (how many of the first, without a gap), which
+// the calling thread and the producer read while the producer (or launcher) writes `published`, and
+// a line shared between writers on different cores would bounce on every update.
 struct alignas(128) HostCounter {
   std::atomic<int> v{0};
 };
@@ -567,11 +568,11 @@ struct alignas(128) HostFlag {
 // most 4096 of them: only requests in flight can complete, so a pass stays as short as the
 // work in flight instead of walking a fixed window of flags.
 void collect(const gsync_serve_cfg* cfg, volatile uint32_t* done, Clock::time_point t0, const int64_t* sched,
-             int64_t* lat, std::atomic<int>* completed, std::atomic<bool>* abort_flag,
+             int64_t* lat, std::atomic<int>* completed, std::atomic<int>* prefix, std::atomic<bool>* abort_flag,
              const std::atomic<int>* published) {
   const int n = cfg->nreq;
   std::vector<char> seen(n, 0);
-  int low = 0, count = 0, reported = 0;
+  int low = 0, count = 0, reported = 0, reported_low = 0;
   while (count < n && !abort_flag->load(std::memory_order_relaxed)) {
     const int hi = std::min(std::min(n, low + 4096), published->load(std::memory_order_acquire));
     for (int q = low; q < hi; ++q) {
@@ -584,6 +585,10 @@ void collect(const gsync_serve_cfg* cfg, volatile uint32_t* done, Clock::time_po
       }
     }
     while (low < n && seen[low]) ++low;
+    if (low != reported_low) {
+      prefix->store(low, std::memory_order_release);
+      reported_low = low;
+    }
     if (count != reported) {  // stored only when it moves, so readers keep the line cached
       completed->store(count, std::memory_order_release);
       reported = count;
@@ -692,13 +697,13 @@ extern "C" int gsync_serve_run(const gsync_serve_cfg* cfg, gsync_serve_buffers* 
   // The loop is running (or about to): publish requests on their schedule, collect completions.
   std::this_thread::sleep_for(std::chrono::microseconds(cfg->start_delay_us));
   const Clock::time_point t0 = Clock::now();
-  HostCounter completed_c, published_c;
+  HostCounter completed_c, prefix_c, published_c;
   HostFlag abort_f;
   std::atomic<int>& completed = completed_c.v;
-  std::atomic<int>& published = published_c.v;
+  std::atomic<int>&prefix = prefix_c.v, &published = published_c.v;
   std::atomic<bool>& abort_flag = abort_f.v;
-  std::thread collector(collect, cfg, buf->done, t0, buf->sched_ns, buf->latency_ns, &completed, &abort_flag,
-                        &published);
+  std::thread collector(collect, cfg, buf->done, t0, buf->sched_ns, buf->latency_ns, &completed, &prefix_c.v,
+                        &abort_flag, &published);
   pin_to_core_from_end(collector, 1);
   const auto deadline = Clock::now() + std::chrono::nanoseconds(buf->sched_ns[cfg->nreq - 1]) +
                         std::chrono::seconds(cfg->drain_timeout_s);
@@ -718,8 +723,9 @@ extern "C" int gsync_serve_run(const gsync_serve_cfg* cfg, gsync_serve_buffers* 
       const int64_t now = now_ns(t0);
       int qe = q + 1;
       while (qe < cfg->nreq && buf->sched_ns[qe] <= now && qe - q < 64) ++qe;
-      // The ring entry of request i is reused only after request i - ring_slots completed.
-      while (qe - 1 - completed.load(std::memory_order_acquire) >= cfg->ring_slots) {
+      // The ring entry of request i is reused only after request i - ring_slots and all before it
+      // completed.  (Requests complete in any order: their number says nothing about one entry.)
+      while (qe - 1 - prefix.load(std::memory_order_acquire) >= cfg->ring_slots) {
         if (Clock::now() > deadline || abort_flag.load(std::memory_order_relaxed)) {
           prod_rc.store(GSYNC_ETIMEDOUT);
           return;
@@ -788,13 +794,13 @@ extern "C" int gsync_serve_baseline(const gsync_serve_cfg* cfg, gsync_serve_buff
   if (int rc = host_dev_ptr(buf->res, &d_res)) return rc;
   if (int rc = host_dev_ptr((void*)buf->done, &d_done)) return rc;
   const Clock::time_point t0 = Clock::now();
-  HostCounter completed_c, published_c;
+  HostCounter completed_c, prefix_c, published_c;
   HostFlag abort_f;
   std::atomic<int>& completed = completed_c.v;
   std::atomic<int>& published = published_c.v;
   std::atomic<bool>& abort_flag = abort_f.v;
-  std::thread collector(collect, cfg, buf->done, t0, buf->sched_ns, buf->latency_ns, &completed, &abort_flag,
-                        &published);
+  std::thread collector(collect, cfg, buf->done, t0, buf->sched_ns, buf->latency_ns, &completed, &prefix_c.v,
+                        &abort_flag, &published);
   pin_to_core_from_end(collector, 1);
   int dev = 0;
   GSYNC_CUDA(cudaGetDevice(&dev));
