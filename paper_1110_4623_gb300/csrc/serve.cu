@@ -720,17 +720,20 @@ extern "C" int gsync_serve_run(const gsync_serve_cfg* cfg, gsync_serve_buffers* 
     int q = 0;
     while (q < cfg->nreq) {
       spin_until(t0 + std::chrono::nanoseconds(buf->sched_ns[q]));
-      const int64_t now = now_ns(t0);
-      int qe = q + 1;
-      while (qe < cfg->nreq && buf->sched_ns[qe] <= now && qe - q < 64) ++qe;
       // The ring entry of request i is reused only after request i - ring_slots and all before it
       // completed.  (Requests complete in any order: their number says nothing about one entry.)
-      while (qe - 1 - prefix.load(std::memory_order_acquire) >= cfg->ring_slots) {
+      int low;
+      while (q - (low = prefix.load(std::memory_order_acquire)) >= cfg->ring_slots) {
         if (Clock::now() > deadline || abort_flag.load(std::memory_order_relaxed)) {
           prod_rc.store(GSYNC_ETIMEDOUT);
           return;
         }
       }
+      // ... of which the ring takes as many as it has room for.
+      const int room = (int)std::min<int64_t>(cfg->nreq, (int64_t)low + cfg->ring_slots);
+      const int64_t now = now_ns(t0);
+      int qe = q + 1;
+      while (qe < room && buf->sched_ns[qe] <= now && qe - q < 64) ++qe;
       for (int i = q; i < qe; ++i) {
         uint64_t* e = (uint64_t*)((char*)buf->ring + (size_t)(i & (cfg->ring_slots - 1)) * kRingStride);
         const uint64_t seq = (uint32_t)(i + 1);
