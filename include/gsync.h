@@ -516,13 +516,18 @@ int gsync_bench_batched(const gsync_batched_work* w, void* stream);
  * after the start and records latency_ns[q] = the host time its completion flag was first
  * seen minus sched_ns[q] (open loop: latency counts from the scheduled arrival).
  *  - On the device, each of the `admitters` blocks admits a batch of nslots / admitters (1 to 8)
- *    requests at a time: it first waits on the admission semaphore (n = nslots in-flight
- *    requests) for a permit each, then takes the batch's indices (its ticket of the ring's
- *    ticket lock), and one warp each waits for a ring entry to be published, claims a free slot
- *    and publishes the request in it; every other block claims chunks of chunk_elems values of
+ *    requests at a time: it takes the batch's indices (its ticket of the ring's ticket lock),
+ *    and one warp each waits on the admission semaphore (n = nslots in-flight requests; the
+ *    index is the request's ticket, so permits go out in the order of the ring and a request
+ *    that takes long keeps only its own), waits for its ring entry to be published, claims a
+ *    free slot and publishes the request in it; every other block claims chunks of chunk_elems values of
  *    any active request; the block that finishes a request's last chunk writes res[q] and
  *    done[q] = 1 into pinned host memory, frees the slot and posts the semaphore.  The
  *    semaphore and the lock are taken before the request arrives, off its latency path.
+ *  - timeout_ns (0 = 2 s) bounds one wait of the loop.  The waits that sparse arrivals make long
+ *    get more: a worker with nothing to do, and the ring lock, 16 times that; a warp of a batch,
+ *    which may wait for the arrivals of all the batches taken before its own, 16 times that for
+ *    each request of a batch (a permit's wait and an entry's wait alike).
  *  - ring (ring_slots entries of 128 bytes, ring_slots a power of two), ctrl (64 words:
  *    ctrl[32] = shutdown), res
  *    (nreq x i64) and done (nreq x u32) are caller-owned pinned host memory

@@ -1768,6 +1768,78 @@ class RingReuse:
         return (0, q), (ring, nxt, done | {q}), None
 
 
+class ServeAdmission:
+    """Admission of a backlog by lanes (the persistent serving loop; not in the paper).
+
+    Block 0 is the worker: it completes any published request of the lowest slot, request `slow`
+    only after all others; it then posts the permit and clears the slot's busy bit, in this order
+    (the device gives the two no order).  Blocks 1.. are the lanes, `lanes` of them to an admitter.  An
+    admitter's first lane takes the next `lanes` indices for all, once every lane is through with
+    the batch before.  A lane waits for its permit (the window's turn plus `slots` past its
+    index), then claims a slot whose busy bit is clear, starting at its index and going on to a
+    free one of the word that the failed attempt returned, and publishes its request there.
+    broken="batch_permits": a lane waits for the permit of its batch's last index (a slow request
+    then keeps the whole next batch out: with slots = lanes nothing behind it completes);
+    broken="blind_set": a lane sets a busy bit without looking whether it was clear.
+    """
+    kind = "mutex"
+    capacity = 1 << 30
+    fifo = False
+
+    def __init__(self, slots=2, lanes=2, requests=5, slow=0, broken=None):
+        self.slots, self.lanes, self.requests, self.slow, self.broken = slots, lanes, requests, slow, broken
+
+    def init(self, nproc, ops):
+        A = (nproc - 1) // self.lanes
+        # shared: batch heads, batches taken and lanes through, by admitter; next index; the
+        # window's turn; busy bits; published request (+ 1) by slot; requests completed
+        sh = ((0,) * A, (0,) * A, (self.lanes,) * A, 0, 0, (0,) * self.slots, (0,) * self.slots, frozenset())
+        return sh, tuple((0, 0, 0, 0) for _ in range(nproc))
+
+    def step(self, p, loc, sh, nproc, ops):
+        heads, taken, through, nxt, turn, busy, slots, done = sh
+        pc, x, h, s = loc
+        R, n = self.requests, self.slots
+        if p == 0:  # worker; x = the slot served
+            if pc == 0:
+                if len(done) == R:
+                    return (DONE, 0, 0, 0), sh, None
+                for i, v in enumerate(slots):
+                    if v and (v - 1 != self.slow or len(done) == R - 1):
+                        return (1, i, 0, 0), sh[:6] + (_set(slots, i, 0), done | {v - 1}), None
+                return loc, sh, None
+            if pc == 1:
+                return (2, x, 0, 0), sh[:4] + (turn + 1,) + sh[5:], None
+            return (0, 0, 0, 0), sh[:5] + (_set(busy, x, 0),) + sh[6:], None
+        a, lane = (p - 1) // self.lanes, (p - 1) % self.lanes  # x = batches this lane has been given
+        if pc == 0:
+            if lane == 0 and taken[a] == x:
+                if through[a] < self.lanes:
+                    return loc, sh, None
+                batch = (_set(heads, a, nxt), _set(taken, a, x + 1), _set(through, a, 0), nxt + self.lanes)
+                return loc, batch + sh[4:], None
+            if taken[a] == x:
+                return loc, sh, None
+            h = heads[a] + lane
+            if h >= R:
+                return (DONE, 0, 0, 0), (heads, taken, _set(through, a, through[a] + 1)) + sh[3:], None
+            return (1, x + 1, h, h % n), sh, None
+        if pc == 1:
+            last = h - lane + self.lanes - 1 if self.broken == "batch_permits" else h
+            if turn + n > last:
+                return (2, x, h, s), sh, None
+            return loc, sh, None
+        if pc == 2:
+            if not busy[s] or self.broken == "blind_set":
+                return (3, x, h, s), sh[:5] + (_set(busy, s, 1),) + sh[6:], None
+            free = [i for i, b in enumerate(busy) if not b]
+            return (2, x, h, free[h % len(free)] if free else s), sh, None
+        if slots[s]:
+            return loc, sh, ("violation", f"request {h} published over request {slots[s] - 1}")
+        out = (heads, taken, _set(through, a, through[a] + 1)) + sh[3:6] + (_set(slots, s, h + 1), done)
+        return (0, x, 0, 0), out, None
+
+
 class ServeSlot:
     """One slot of the persistent serving loop (not in the paper): an admitter publishes
     requests into the slot one after another, and workers claim the requests' chunks.

@@ -8,11 +8,11 @@
 // link, or managed memory placed in device memory, which the host writes in place and the
 // admitters poll through L2.  Inside one co-resident
 // launch:
-//   * admitter blocks admit a batch of requests at a time, one per warp: they wait on the
-//     admission semaphore (n = number of in-flight slots) for a permit each, take the batch's
-//     request indices with one acquisition of the ring's ticket lock, and each warp waits for its
-//     entry to appear, claims a free slot and publishes the request in it (release store of the
-//     slot's claim word);
+//   * admitter blocks admit a batch of requests at a time, one per warp: they take the batch's
+//     request indices with one acquisition of the ring's ticket lock, and each warp waits on the
+//     admission semaphore (n = number of in-flight slots) for its request's permit, waits for
+//     its entry to appear, claims a free slot and publishes the request in it (release store of
+//     the slot's claim word);
 //   * every other block claims chunks of any active slot (fetch-and-add on the slot's claim
 //     word), sums the chunks' int32 values in int64 until the request has
 //     none left to hand out, and adds its partial to the slot's accumulator; the block that
@@ -193,53 +193,53 @@ __device__ __forceinline__ void lanes_sync(uint32_t lanes) {
   asm volatile("barrier.sync 1, %0;" ::"r"(lanes * 32u) : "memory");
 }
 
-// Takes `n` permits of the ticket-window semaphore at once (n at most its count): n tickets in
-// a row, entered when the last of them is admitted.  Tickets are admitted in order, so at
-// most one caller holds some of its permits while it waits for the others.
-__device__ __forceinline__ int window_wait_many(const gsync::SemRef& s, uint32_t n) {
-  const uint32_t last = ptx::atom_add_relaxed(s.word(1), n) + n - 1u;
-  gsync::Waiter w;
-  uint32_t turn = ptx::ld_acquire(s.word(2));
-  while (!gsync::after(turn + s.n, last)) {
-    if (int rc = w.tick(s.timeout_ns, s.abort_word())) return rc;
-    const uint32_t ahead = last - (turn + s.n) + 1u;
-    if (s.bo.min_ns && ahead < 0x80000000u) {
-      const uint32_t ns = ahead * s.bo.min_ns;
-      gsync::sleep_to_poll(ns < s.bo.max_ns ? ns : s.bo.max_ns);
-    }
-    turn = ptx::ld_acquire(s.word(2));
-  }
-  return GSYNC_OK;
-}
-__device__ __forceinline__ void window_post_many(const gsync::SemRef& s, uint32_t n) {
-  ptx::red_add_release(s.word(2), n);
-}
-
-// Thread 0 of an admitter: a permit and a ring index for each lane, or false to stop.
-__device__ __forceinline__ bool take_indices(const Args& a, const gsync::SemRef& sem, const gsync::MutexRef& lock,
-                                             uint32_t& head) {
+// Thread 0 of an admitter: the next batch of ring indices, one for each lane.  The ring lock's
+// tickets are handed out in order from 0, one per acquisition, so ticket t stands for the indices
+// t * lanes .. + lanes - 1: the holder needs no head word and releases the lock at once, and as
+// the lock hands on nothing but the ticket itself, the release needs no fence.
+__device__ __forceinline__ bool take_indices(const Args& a, const gsync::MutexRef& lock, uint32_t& head) {
   if (ptx::ld_relaxed(a.dev_shutdown)) return false;
-  const int rc = window_wait_many(sem, a.lanes);
-  if (rc != GSYNC_OK) {
-    record_status(a.status, rc);
-    return false;
-  }
-  if (ptx::ld_relaxed(a.dev_shutdown)) {  // pass the permits on so blocked admitters exit too
-    window_post_many(sem, a.lanes);
-    return false;
-  }
-  // The ring lock's tickets are handed out in order from 0, one per acquisition, so ticket t
-  // stands for the indices t * lanes .. + lanes - 1: the holder needs no head word and releases
-  // the lock at once.
   const gsync::Token t = gsync::mutex_lock_thread<GSYNC_MUTEX_TICKET>(lock);
   if (t.status != GSYNC_OK) {
     record_status(a.status, t.status);
     return false;
   }
-  // The lock hands on nothing but the ticket itself, so its release needs no fence.
   ptx::st_relaxed(lock.turn(), t.ticket + 1u);
   head = t.ticket * a.lanes;
   return true;
+}
+
+// The shutdown word that the host sets, looked at by one of the lanes and passed on to all.
+__device__ __forceinline__ bool host_shutdown(const Args& a) {
+  if (!ld_acquire_sys(a.shutdown)) return false;
+  ptx::st_release(a.dev_shutdown, 1u);
+  return true;
+}
+
+// One lane: waits for a permit of the admission semaphore.  Every request takes one permit and one
+// index, so the index is also its ticket of the window: request h enters once h - nslots + 1
+// requests have completed.  Each lane enters by itself, so a request that takes long keeps one
+// slot from the others, and not the batch behind it (a batch that entered with its last ticket waited
+// for the whole one before with slots = lanes: 8 slots, 1 admitter, 7 of 8 slots empty beside a long
+// request); and permits go out in the order of the ring, also where the ring is shorter than the
+// indices taken.  False to stop.
+__device__ __forceinline__ bool wait_permit(const Args& a, const gsync::SemRef& s, uint32_t h) {
+  gsync::Waiter w;
+  uint32_t polls = 0;
+  for (;;) {
+    const uint32_t turn = ptx::ld_acquire(s.word(2));
+    if (gsync::after(turn + s.n, h)) return true;
+    // the bound of one permit's wait, for each of the batch that a lane may wait behind
+    if (int rc = w.tick(s.timeout_ns * a.lanes, s.abort_word())) {
+      record_status(a.status, rc);
+      return false;
+    }
+    ++polls;
+    if ((polls & 7u) == 0u && ptx::ld_relaxed(a.dev_shutdown)) return false;
+    if ((polls & 255u) == 0u && host_shutdown(a)) return false;
+    const uint32_t ns = (h - (turn + s.n) + 1u) * s.bo.min_ns;
+    gsync::sleep_to_poll(ns < s.bo.max_ns ? ns : s.bo.max_ns);
+  }
 }
 
 // Claims a slot whose bit is clear in the busy word, h mod nslots if that one is free.  The atomic
@@ -282,10 +282,11 @@ __device__ __forceinline__ void retire_slot(const Args& a, uint32_t s) {
   for (uint32_t k = 0; k < kMaskCopies; ++k) atomicAnd(&a.active_mask[32u * k + (s >> 5)], ~(1u << (s & 31)));
 }
 
-// One lane: waits for ring entry h (seq == seq_check == h + 1), claims a free slot and
-// publishes the request in it.  False to stop (shutdown, or a wait that ran out).
+// One lane: waits for a permit and for ring entry h (seq == seq_check == h + 1), claims a free slot
+// and publishes the request in it.  False to stop (shutdown, or a wait that ran out).
 __device__ __forceinline__ bool admit(const Args& a, const gsync::SemRef& sem, uint32_t h) {
   const gsync_serve_req* e = (const gsync_serve_req*)((const char*)a.ring + (size_t)(h & a.ring_mask) * kRingStride);
+  if (!wait_permit(a, sem, h)) return false;
   uint64_t lo, hi;  // seq | len << 32 and off | seq_check << 32
   uint32_t polls = 0;
   const uint64_t t0 = ptx::globaltimer();
@@ -293,17 +294,10 @@ __device__ __forceinline__ bool admit(const Args& a, const gsync::SemRef& sem, u
     ld_acquire_sys_v2(e, lo, hi);
     if ((uint32_t)lo == h + 1u && (uint32_t)(hi >> 32) == h + 1u) break;
     if ((++polls & 15u) == 0) {
-      bool stop = false;
-      if (ld_acquire_sys(a.shutdown)) {
-        ptx::st_release(a.dev_shutdown, 1u);
-        stop = true;
-      } else if (ptx::globaltimer() - t0 > a.timeout_ns * 16 * a.lanes) {
+      if (host_shutdown(a)) return false;
+      if (ptx::globaltimer() - t0 > a.timeout_ns * 16 * a.lanes) {
         // the bound of one entry's wait, for each of the batch that a lane may wait behind
         record_status(a.status, GSYNC_ETIMEDOUT);
-        stop = true;
-      }
-      if (stop) {  // the permit goes back so that admitters blocked on it can see shutdown
-        gsync::sem_post_thread<GSYNC_SEM_WINDOW>(sem);
         return false;
       }
     }
@@ -345,8 +339,8 @@ __global__ void __launch_bounds__(kThreads, 3) serve_kernel(Args a) {
   uint64_t idle_since = 0;
 
   if (admitter) {
-    // Admitters: semaphore -> ring indices (ticket lock) -> wait for those entries -> slots.
-    // The permits and the indices are taken before the requests exist, so an arrival only
+    // Admitters: ring indices (ticket lock) -> permits -> wait for those entries -> slots.
+    // The indices and the permits are taken before the requests exist, so an arrival only
     // waits for one read of host memory.  A block admits `lanes` requests at a time, lane w
     // (thread 0 of warp w) the w-th of them.  What bounds a backlog is the ring lock's chain of
     // hand-offs: with one acquisition per request it took 0.83 us a request whatever the number
@@ -357,7 +351,7 @@ __global__ void __launch_bounds__(kThreads, 3) serve_kernel(Args a) {
     if (lane >= a.lanes) return;
     if (tid == 0) s_left = 0;
     for (;;) {
-      if (tid == 0) s_taken = take_indices(a, sem, lock, s_head) ? 1 : 0;
+      if (tid == 0) s_taken = take_indices(a, lock, s_head) ? 1 : 0;
       lanes_sync(a.lanes);
       if (!s_taken) return;
       if ((tid & 31u) == 0u && !admit(a, sem, s_head + lane)) s_left = 1;
@@ -643,8 +637,8 @@ extern "C" int gsync_serve_run(const gsync_serve_cfg* cfg, gsync_serve_buffers* 
   uint32_t* status = (uint32_t*)p;    p += 128;
   uint32_t* dev_shutdown = (uint32_t*)p;
   GSYNC_CUDA(cudaMemsetAsync(workspace, 0, gsync_serve_workspace_bytes(cfg->nslots), st));
-  // Admitters may legitimately wait for a permit or an index while arrivals are sparse: the
-  // lock and the semaphore get 16x the per-wait bound.
+  // Admitters may legitimately wait for a permit while arrivals are sparse (more admitters than
+  // slots): the lock and the semaphore get 16x the per-wait bound.
   const uint64_t wait_ns = (cfg->timeout_ns ? cfg->timeout_ns : 2000000000ull) * 16;
   if (int rc = gsync_mutex_init(ring_lock, 3 * 128, GSYNC_MUTEX_TICKET, 1, nullptr, wait_ns, stream)) return rc;
   gsync_backoff sbo = {GSYNC_BACKOFF_EXPONENTIAL, 64, 2000, 0};
