@@ -14,10 +14,10 @@
 //     its entry to appear, claims a free slot and publishes the request in it (release store of
 //     the slot's claim word);
 //   * every other block claims chunks of any active slot (fetch-and-add on the slot's claim
-//     word), sums the chunks' int32 values in int64 until the request has
-//     none left to hand out, and adds its partial to the slot's accumulator; the block that
-//     finishes a request writes the result and a completion flag into pinned host memory,
-//     frees the slot and posts the semaphore.
+//     word), sums the chunks' int32 values in int64 (with a backlog, a bounded run of one
+//     request's), and adds its partial to the slot's accumulator; the block that finishes a
+//     request writes the result and a completion flag into pinned host memory, frees the
+//     slot and posts the semaphore.
 // Requests that arrive while others run are admitted as slots free up and their chunks run
 // side by side with older requests' chunks.  Every wait is bounded (the object timeouts, or
 // the loop's own deadline) and the host's shutdown word ends the loop.
@@ -58,6 +58,12 @@ constexpr uint32_t kMaskCopies = 4;
 // Active slots from which a worker goes on with the chunks of the request it has: at 1e6 req/s
 // about seven requests are in flight, a drained backlog keeps most slots active.
 constexpr int kBacklog = 8;
+// ... and the most chunks it takes of one request before it looks at the others again: a worker that
+// stayed until the request had no more left was lost to the short requests beside a long one (64
+// slots, 3 workers, 600 requests of one chunk beside one of 30,000: the short ones done after 12.3 ms
+// instead of 0.9).  At 16 a backlog of 3000 requests in chunks of 2048 takes as long as without a
+// limit (3.58 and 3.59 ms), at 8 as well (3.61), at 4 3.72.
+constexpr uint32_t kKeep = 16;
 
 struct Slot {  // one 128-byte line
   // The claim word: chunk count << 32 | next chunk to hand out.  Only ever read, added to and
@@ -419,7 +425,7 @@ __global__ void __launch_bounds__(kThreads, 3) serve_kernel(Args a) {
     const int cmd = s_cmd;
     if (cmd == 1) break;
     if (cmd == 2) { __syncthreads(); continue; }
-    // With a backlog, chunks of this request until they are all handed out, added up in registers:
+    // With a backlog, up to kKeep chunks of this request in a row, added up in registers:
     // one reduction and one count of done chunks per block and request (with few requests in
     // flight other blocks are free, and a chunk taken early would only wait here).  Thread 0 asks
     // for the next one
@@ -430,7 +436,8 @@ __global__ void __launch_bounds__(kThreads, 3) serve_kernel(Args a) {
     uint32_t taken = 0;
     for (uint32_t k = 0;; k ^= 1u) {
       uint32_t next = nchunks;
-      if (tid == 0 && backlog && chunk + 1u < nchunks) next = (uint32_t)ptx::atom_add_relaxed_u64(&sl->claim, 1ull);
+      if (tid == 0 && backlog && taken + 1u < kKeep && chunk + 1u < nchunks)
+        next = (uint32_t)ptx::atom_add_relaxed_u64(&sl->claim, 1ull);
       sum += thread_sum(a.pool, s_lo[k], s_hi[k]);
       ++taken;
       if (tid == 0) {
