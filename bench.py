@@ -142,6 +142,27 @@ def result_rows(out):
     return [dict(row, **stamp) for row in rows]
 
 
+# The keys of the full record that the printed line repeats as they are.
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+             "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks", "roofline", "cpu_baseline",
+             "p99_latency_us", "parity_after_timing", "wall_s_timed_loop")
+
+
+def headline(out):
+    """The line printed on stdout: the record's headline keys and, instead of its sections, one figure
+    per measured configuration (the sections come to 30 KB, more than a reader of the last lines
+    of a log gets)."""
+    figures = {}
+    for row in result_rows(out):
+        if row["section"].startswith("sweep"):
+            continue
+        name = [row["section"], row["kind"]]
+        name += [f"{k}={row[k]:g}" for k in ("cs_words", "n", "offered_req_s") if k in row]
+        unit = next(k for k in ("acq_per_s", "ns_per_crossing", "ops_per_s", "items_per_s", "p99_us") if k in row)
+        figures.setdefault(unit, {})[" ".join(name)] = float(f"{row[unit]:.5g}")
+    return dict({k: out[k] for k in LINE_KEYS if k in out}, figures=figures)
+
+
 def dist_env():
     rank = int(os.environ.get("RANK", "0"))
     world = int(os.environ.get("WORLD_SIZE", "1"))
@@ -1016,7 +1037,8 @@ def run_gpu(args):
             with open(args.jsonl, "a") as f:
                 for row in result_rows(out):
                     f.write(json.dumps(row, default=float) + "\n")
-        print(json.dumps(out, default=float))
+        print("full record:", json.dumps(out, default=float), file=sys.stderr, flush=True)
+        print(json.dumps(headline(out), default=float))
     if world > 1:
         torch.distributed.destroy_process_group()
 
