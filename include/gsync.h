@@ -116,7 +116,9 @@ enum {
 
 typedef struct gsync_backoff {
   uint32_t policy; /* GSYNC_BACKOFF_* */
-  uint32_t min_ns; /* first sleep (and, for ticket locks, sleep per waiter ahead); 0 = no sleeping */
+  uint32_t min_ns; /* first sleep (and, for ticket locks and the TICKET and WINDOW semaphores, sleep
+                      per waiter ahead); 0 = no sleeping.  The semaphores poll at once where waiters
+                      ahead x min_ns is 64 ns or less: a sleep that short takes as long as longer ones */
   uint32_t max_ns; /* cap */
   uint32_t spin;   /* SPIN_THEN_SLEEP: failed attempts before the first sleep (0 selects 32) */
 } gsync_backoff;
@@ -188,7 +190,8 @@ int gsync_device_topology(uint8_t* die_of_sm, int* ndies_out, void* stream);
  * FLAG takes at most 8192 blocks), number of arrival counters (SHARDED, 1..32), S | R << 8
  * (SPLIT: S arrival counters and R release copies, 1..64 each), 0 or 1 (DIE: per-die counters,
  * or one flat counter with a release word on each die), sleep | S << 16 (COUNT: sleep 0..1023 =
- * ns of sleep before the first poll per 16 arrivals still missing, 0 polls at once; S 0..64,
+ * ns of sleep before the first poll per 16 arrivals still missing, 0 polls at once, as does a
+ * sleep that comes to 64 ns or less (CLUSTER and EXCHANGE alike); S 0..64,
  * S > 1 counts in through S sub-counters), 0 (ATOMIC).  FLAG and SHARDED need blockDim.x >= 32 (warp 0 of block 0 gathers the arrivals).
  * DIE takes 32 KB; its init measures the SM-to-die map and the home die of the state's
  * 4 KB pages as gsync_mutex_init_cohort does (and synchronizes `stream`); the first

@@ -313,14 +313,21 @@ struct Backoff {
   }
 };
 
-// Sleep before the next poll, for `ns` that a barrier or a semaphore worked out from what is still
-// missing.  __nanosleep takes 40-65 ns whatever less is asked for, a third of a poll's round trip:
-// a wait that short is better spent polling.  (Ticket window, 16 ns per holder ahead: 1184 blocks,
-// n = 16, 236,800 pairs 34.7 -> 34.2 ms, 344 blocks, n = 6, 9976 pairs 2.18 -> 2.14 ms; counting barrier,
-// 8 ns per 16 arrivals missing: 1.63 -> 1.59 us a crossing at 148 blocks, 1.62 -> 1.60 at 16, and 2.06
-// at 1184 as before; exchange barrier 1.22 -> 1.18 us at 148.)
-__device__ __forceinline__ void sleep_to_poll(uint32_t ns) {
-  if (ns > 64u) __nanosleep(ns);
+// Sleep before the next poll: `ns` is what a barrier or a semaphore worked out from what is still
+// missing, max_ns the cap.  __nanosleep takes 40-65 ns whatever less is asked for, a third of a poll's
+// round trip: a wait that short is better spent polling.  The line is drawn at the wait itself, not
+// at what the cap leaves of it: a cap of 64 ns or less still paces a long queue (window, 1184 blocks,
+// n = 16, cap 48 ns, 35,520 pairs: 5.45 ms, 5.65 without its sleeps).  (Ticket window, 16
+// ns per holder ahead: 1184 blocks, n = 16, 236,800 pairs 34.7 -> 34.2 ms, 344 blocks, n = 6, 9976
+// pairs 2.18 -> 2.14 ms; counting barrier, 8 ns per 16 arrivals missing: 1.63 -> 1.59 us a crossing
+// at 148 blocks, 1.62 -> 1.60 at 16, and 2.06 at 1184 as before; exchange barrier 1.22 -> 1.18 us
+// at 148.)
+constexpr uint32_t kPollInstead = 64u;
+__host__ __device__ constexpr uint32_t poll_sleep_ns(uint32_t ns, uint32_t max_ns) {
+  return ns <= kPollInstead ? 0u : ns < max_ns ? ns : max_ns;
+}
+__device__ __forceinline__ void sleep_to_poll(uint32_t ns, uint32_t max_ns) {
+  if (const uint32_t t = poll_sleep_ns(ns, max_ns)) __nanosleep(t);
 }
 
 __device__ __forceinline__ uint64_t header_timeout(const uint32_t* s) {
@@ -868,7 +875,7 @@ __device__ __forceinline__ int sem_wait_thread(const SemRef& s) {
       const uint32_t ahead = wi - turn;
       if (s.bo.min_ns && ahead < 0x80000000u) {
         const uint32_t ns = ahead * s.bo.min_ns;
-        sleep_to_poll(ns < s.bo.max_ns ? ns : s.bo.max_ns);
+        sleep_to_poll(ns, s.bo.max_ns);
       }
     }
     return GSYNC_OK;
@@ -884,7 +891,7 @@ __device__ __forceinline__ int sem_wait_thread(const SemRef& s) {
       const uint32_t ahead = t - (turn + s.n) + 1u;
       if (s.bo.min_ns && ahead < 0x80000000u) {
         const uint32_t ns = ahead * s.bo.min_ns;
-        sleep_to_poll(ns < s.bo.max_ns ? ns : s.bo.max_ns);
+        sleep_to_poll(ns, s.bo.max_ns);
       }
       turn = ptx::ld_acquire(s.word(2));
     }
@@ -1268,7 +1275,7 @@ __device__ __forceinline__ int barrier_wait(BarrierRef& b) {
         // off the counter while the atomic unit works through the rest of the arrivals.
         if (sleep16 && missing < (1ull << 24)) {
           const uint64_t ns = missing * sleep16 / 16u;
-          sleep_to_poll((uint32_t)(ns < 4000u ? ns : 4000u));
+          sleep_to_poll((uint32_t)ns, 4000u);
         }
       }
       if (S > 1u || missing) {
@@ -1304,7 +1311,7 @@ __device__ __forceinline__ int barrier_wait(BarrierRef& b) {
           const uint32_t sleep16 = (b.param >> 8) & 0x3FFu;
           if (missing && sleep16 && missing < (1ull << 24)) {
             const uint64_t ns = missing * sleep16 / 16u;
-            sleep_to_poll((uint32_t)(ns < 4000u ? ns : 4000u));
+            sleep_to_poll((uint32_t)ns, 4000u);
           }
         }
         int rc = GSYNC_OK;
@@ -1511,7 +1518,7 @@ __device__ __forceinline__ int barrier_exchange(BarrierRef& b, uint64_t value) {
     if (missing) {
       if (sleep16 && missing < (1ull << 24)) {
         const uint64_t ns = missing * sleep16 / 16u;
-        sleep_to_poll((uint32_t)(ns < 4000u ? ns : 4000u));
+        sleep_to_poll((uint32_t)ns, 4000u);
       }
       Waiter w;
       while (ptx::ld_relaxed_u64(counter) < target)

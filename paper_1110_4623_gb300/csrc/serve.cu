@@ -244,7 +244,7 @@ __device__ __forceinline__ bool wait_permit(const Args& a, const gsync::SemRef& 
     if ((polls & 7u) == 0u && ptx::ld_relaxed(a.dev_shutdown)) return false;
     if ((polls & 255u) == 0u && host_shutdown(a)) return false;
     const uint32_t ns = (h - (turn + s.n) + 1u) * s.bo.min_ns;
-    gsync::sleep_to_poll(ns < s.bo.max_ns ? ns : s.bo.max_ns);
+    gsync::sleep_to_poll(ns, s.bo.max_ns);
   }
 }
 
