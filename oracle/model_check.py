@@ -38,8 +38,11 @@ The algorithms follow Section 5 ("Design") and the pseudocode of the Appendix:
   SplitBarrier  S arrival counters under a top counter, R copies of the release word
   CountBarrier  one growing arrival counter that every block polls
   ExchangeBarrier  the counting barrier whose arrivals carry one value per block, no fence
+  FullFold      the barrier workload's late full fold, over crossings that fail
   RingPublish   the serving ring's entry, written as two single-copy-atomic halves, no fence
-  ServeSlot     a serving slot: generation-tagged chunk claims by fetch-and-add, reuse
+  RingReuse     the reuse of the ring's entries, by the completed prefix
+  ServeAdmission  admission by lanes: permits by ring index, the busy word
+  ServeSlot     a serving slot: chunk claims by fetch-and-add on one claim word, reuse
 Mutation variants with a planted mistake (`broken=...`) exist so that tests can show the
 checker catches each kind of error.
 """
@@ -1668,6 +1671,49 @@ class ClusterCountBarrier:
 # --------------------------------------------------------------------------------------------
 # Explorer
 # --------------------------------------------------------------------------------------------
+
+
+class FullFold:
+    """The barrier workload's full fold in one block (not in the paper): the warps' shares of a round
+    lie in two halves by round parity, and warp 0 puts them together one round late.
+
+    Block 0 is warp 0, blocks 1.. are the block's other warps.  `ok[r]` says whether crossing r
+    succeeds (all warps learn the same).  After crossing r, which all warps pass together, warp 0
+    puts the pending round together, which reads the other warps' shares one by one, and then every
+    warp writes its share of round r; a failed crossing has no shares, and warp 0 puts the pending
+    round together before it goes on.
+    broken="kept_pending": it keeps the pending round over the failed crossing instead (and reads
+    the half that the others write after the next one).
+    """
+    kind = "mutex"
+    capacity = 1
+    fifo = False
+
+    def __init__(self, ok=(1, 1, 0, 1, 1), broken=None):
+        self.ok, self.broken = ok, broken
+
+    def init(self, nproc, ops):
+        # shared: (crossings reached per warp, the halves' shares by warp); local: (pc, r, pending, warp)
+        return ((0,) * nproc, ((-1,) * nproc,) * 2), tuple((0, 0, -1, 0) for _ in range(nproc))
+
+    def step(self, p, loc, sh, nproc, ops):
+        pc, r, pend, w = loc
+        reached, red = sh
+        if pc == 0:  # arrives at crossing r
+            return (1, r, pend, 0), (_set(reached, p, r + 1), red), None
+        if pc == 1:
+            if min(reached) <= r:
+                return loc, sh, None
+            fold = p == 0 and pend >= 0 and (self.ok[r] or self.broken != "kept_pending")
+            return ((2 if fold else 3), r, pend, 0), sh, None
+        if pc == 2:  # warp w's share of the pending round
+            if red[pend & 1][w] != pend:
+                return loc, sh, ("violation", f"round {pend} put together with a share of round {red[pend & 1][w]}")
+            return ((2, r, pend, w + 1) if w + 1 < nproc else (3, r, -1, 0)), sh, None
+        if self.ok[r]:
+            red = _set(red, r & 1, _set(red[r & 1], p, r))
+            pend = r
+        return ((0 if r + 1 < len(self.ok) else DONE), r + 1, pend, 0), (reached, red), None
 
 
 class RingPublish:
