@@ -52,8 +52,8 @@ enum {
 
 /* Mutex kinds (Section 5, "Mutex"; Appendix, spin-lock and FA mutex pseudocode). */
 typedef enum gsync_mutex_kind {
-  GSYNC_MUTEX_CAS_SPIN = 0,    /* spin on atomicCAS(0 -> 1), paced in grids that would fill the
-                                  atomic unit (above 676 blocks); unlock = release store 0 */
+  GSYNC_MUTEX_CAS_SPIN = 0,    /* spin on atomicCAS(0 -> 1), paced in grids that could fill
+                                  the atomic unit (from 680 blocks on); unlock = release store 0 */
   GSYNC_MUTEX_CAS_BACKOFF = 1, /* the same with __nanosleep backoff after each failure */
   GSYNC_MUTEX_TICKET = 2,      /* fetch-and-add ticket; poll turn; unlock stores turn + 1 */
   GSYNC_MUTEX_SLEEP_QUEUE = 3, /* queue lock: each waiter polls its own padded flag slot */

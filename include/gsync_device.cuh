@@ -466,19 +466,35 @@ enum : uint32_t { kCohortOwned = 0x80000000u };
 // CLUSTER_MCS record: bit 16 says the cluster already holds the global lock.
 constexpr uint64_t kMcsOwned = 1ull << 16;
 
-// CAS_SPIN: pause between two attempts (ns, 0 = none).  Every block that spins asks the lock's
+// CAS_SPIN: the pause between two attempts (ns, 0 = none).  Every block that spins asks the lock's
 // atomic unit for one swap per round trip, and the unlock's store queues behind them.  The unit
 // takes a same-word swap each ~0.65 ns and an unloaded round trip is ~400 ns, so it is full from
 // about 620 blocks on.  A larger grid spaces each block's attempts to one per (blocks x 0.65 ns)
 // round, the unit's own pace: enough that some block tries every ns, and no queue.  1184 blocks x
 // 256 threads, 64-word section, 100 acquisitions each: 229 -> 145 ms (516 -> 815 K/s); 20 each: 900
 // blocks 23.3 -> 19.2 ms, 700 blocks 15.6 -> 14.6.
-// Up to 676 blocks there is no pause, and the loop is the plain one (at 592 a pause gains 1 %).
+// Below 680 blocks there is no pause, and the loop is the plain one (at 592 a pause gains 1 %).
 // Spinning on a load between attempts instead lets every waiter see the lock free at once: 1.17x
 // at 1184 blocks where the pause gives 1.42x (30 each).
-__device__ __forceinline__ uint32_t cas_spin_pause_ns() {
-  const uint32_t round_ns = gridDim.x * gridDim.y * gridDim.z / 20u * 13u;
-  return round_ns > 440u ? min(round_ns - 400u, 4000u) : 0u;
+// The grid is only the most that the lock can be wanted by: it may be larger than what is resident,
+// or spread over many locks.  So the first four attempts come at once, and a waiter's pause starts at
+// no more than what 1200 blocks call for (380 ns) and reaches a larger grid's only by 8 ns an attempt,
+// for a lock that many must be waiting for.  100,000 acquisitions by blocks of 256 threads with nothing
+// else to do, ms without a pause / with the whole grid's from the fifth attempt / so: 4864 blocks, 256
+// locks 0.46 / 0.74 / 0.56, 2048 locks 0.125 / 0.153 / 0.125; 20,000 blocks, one lock 983 / 126 / 111.
+// What is left of the price is at locks that few blocks want in a grid this large: 1216 blocks, 256
+// locks 0.52 / 0.58 / 0.58, 16 locks 5.8 / 6.6 / 6.6; where the blocks also load and store under the lock a
+// pause still gains (1184 blocks of 128, 200,000 acquisitions of the batched kernel: 64 keys 7.4 /
+// 6.3 / 6.3, 256 keys 2.4 / 2.2 / 2.2, 4096 keys 0.35 / 0.34 / 0.34).
+constexpr uint32_t kSpinFirst = 4u;  // attempts without a pause: a lock few blocks want is free by then
+__host__ __device__ constexpr uint32_t cas_spin_most_ns(uint32_t blocks) {
+  const uint32_t round_ns = blocks / 20u * 13u;
+  return round_ns <= 440u ? 0u : round_ns < 4400u ? round_ns - 400u : 4000u;
+}
+__host__ __device__ constexpr uint32_t cas_spin_pause_ns(uint32_t most_ns, uint32_t polls) {
+  const uint32_t grown = polls < 512u ? polls * 8u : 4096u;
+  const uint32_t ns = grown > 380u ? grown : 380u;
+  return polls <= kSpinFirst ? 0u : ns < most_ns ? ns : most_ns;
 }
 
 // Master-thread lock.  Returns the ticket (ticket kinds) in tok.ticket.
@@ -491,10 +507,10 @@ __device__ __forceinline__ Token mutex_lock_thread(const MutexRef& m) {
     uint32_t sleep_ns = m.bo.min_ns;
     uint32_t spins = m.bo.policy == GSYNC_BACKOFF_SPIN_THEN_SLEEP ? m.bo.spin : 0u;
     if (KIND == GSYNC_MUTEX_CAS_SPIN) {
-      if (const uint32_t pause = cas_spin_pause_ns()) {
+      if (const uint32_t most = cas_spin_most_ns(gridDim.x * gridDim.y * gridDim.z)) {
         while (ptx::atom_cas_acquire(m.lockw(), 0u, 1u) != 0u) {
           if (int rc = w.tick(m.timeout_ns, m.abort_word())) return {rc, 0u};
-          if (w.polls > 4u) __nanosleep(pause);  // a lock few blocks want is free by then
+          if (const uint32_t pause = cas_spin_pause_ns(most, w.polls)) __nanosleep(pause);
         }
         return {GSYNC_OK, 0xFFFFFFFFu};
       }
