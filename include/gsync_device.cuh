@@ -916,9 +916,10 @@ __device__ __forceinline__ int sem_wait_thread(const SemRef& s) {
     uint32_t sleep_ns = s.bo.min_ns;
     for (;;) {
       // SPIN looks before it swaps: a waiter that swaps a word with no permit in it keeps the
-      // posts out for two atomic round trips (148 blocks, n = 4: 5.36 -> 0.82 ms for 740 pairs).
-      // SPIN_BACKOFF swaps at once: its sleeps keep the word free enough, and a look would add a
-      // round trip to the attempts that do find a permit (296 blocks, n = 4: 5.9 against 8.4 ms).
+      // posts out for two atomic round trips (148 blocks, n = 4: 5.36 -> 1.11 ms for 740 pairs; 0.83
+      // with the post's fence before its swap).  SPIN_BACKOFF swaps at once: its sleeps keep the word
+      // free enough, and a look would add a round trip to the attempts that do find a permit (296
+      // blocks, n = 4, 5920 pairs: 8.4 ms with a look, 5.7 without).
       if (KIND == GSYNC_SEM_SPIN_BACKOFF || ptx::ld_relaxed(s.word(1)) > 1u) {
         const uint32_t v = ptx::atom_exch_acquire(s.word(1), 0u);
         if (v > 1u) {
@@ -950,7 +951,7 @@ __device__ __forceinline__ int sem_post_thread(const SemRef& s) {
   } else {
     // The release's fence comes before the swap, not between it and the new value: while the word
     // is 0 every other wait and post stands still, and the fence is the longer part of that time
-    // (296 blocks, n = 4, backoff: 8.4 -> 5.9 ms for 5920 pairs).
+    // (296 blocks, n = 4, 5920 pairs: with backoff 8.0 -> 5.7 ms, without 8.6 -> 6.5).
     ptx::fence_acq_rel();
     Waiter w;
     for (;;) {

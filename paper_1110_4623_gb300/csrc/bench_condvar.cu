@@ -21,8 +21,9 @@ struct __align__(16) Queue {
 // ROOMY: up to 48 registers a thread.  Left to itself the ticket lock's kernel takes 32, which lets
 // 2432 blocks of 128 threads be resident, and keeps some of thread 0's state in local memory: every
 // acquire empties L1, so each look at it under the lock is an L2 round trip.  The roomy form runs
-// where its smaller limit (1520) admits the grid (592 + 592 blocks, 5920 items, on new states 20.4 ->
-// 19.4 ms, on states run before 19.6 -> 19.4; 384 + 384 of 32 threads 10.45 -> 10.33; 128 + 64 6.90 -> 6.85).
+// where its smaller limit (1520) admits the grid (592 + 592 blocks, 5920 items, medians of 18 new states
+// 19.6 -> 19.1 ms, of their later runs 19.1 -> 18.8, single ones 18.2 to 22; 384 + 384 of 32 threads 10.45
+// -> 10.33; 128 + 64 6.90 -> 6.85).
 template <int MKIND, bool ROOMY = false>
 __global__ void __launch_bounds__(kMaxThreads, ROOMY ? 5 : 0)
     condvar_workload_kernel(uint32_t* mutex_state, uint32_t* nf_state, uint32_t* ne_state, Queue* q, uint32_t* buf,

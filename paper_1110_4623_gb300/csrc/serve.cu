@@ -428,8 +428,8 @@ __global__ void __launch_bounds__(kThreads, 3) serve_kernel(Args a) {
     // With a backlog, up to kKeep chunks of this request in a row, added up in registers:
     // one reduction and one count of done chunks per block and request (with few requests in
     // flight other blocks are free, and a chunk taken early would only wait here).  Thread 0 asks
-    // for the next one
-    // before it sums its share of this one, so the claim's round trip passes under the loads.
+    // for the next one before it sums its share of this one, so the claim's round trip passes
+    // under the loads.
     // No other request can take the slot meanwhile (this block's chunks are not counted done),
     // so the claim needs no look at the slot, and a claim past the last chunk ends it.
     long long sum = 0;
